@@ -54,7 +54,14 @@ struct FwdCfg {
   static constexpr int BM = kPlan.bm;         // rows per query tile (= TMEM lanes)
   static constexpr int NQT = kPlan.q_tiles;   // query tiles per CTA
   static constexpr int BN = kPlan.bn;         // keys per KV tile
-  static constexpr int NSLOT = SLOTS ? SLOTS : kPlan.kv_slots;  // K/V ring slots
+  // At D = 128 both query tiles stage their O in one 32 KB block, in turn (see
+  // softmax_epilogue), and the 32 KB this frees are one more ring slot than the plan's 3: with
+  // three slots the MMA warp waited for K of every tile (about 300 of a pair of tile-steps'
+  // 2700 clocks in a clock trace).  GB300, same box, three slots against four: B4 H32 S2048
+  // 190.7 -> 185.2 us, causal 116.9 -> 113.0, ragged causal batch (16 sequences of 1024 to
+  // 8192) 2389 -> 2351.  D = 64 has ten slots and a block per tile.
+  static constexpr bool SHARED_STG = D == 128;
+  static constexpr int NSLOT = SLOTS ? SLOTS : kPlan.kv_slots + (SHARED_STG ? 1 : 0);  // K/V ring slots
   static_assert(BM == 128 && NQT == 2, "warp roles assume two 128-row query tiles");
   static_assert(BN == 128, "softmax holds one S row of 128 fp32 in registers, P leaves in two 64-key halves");
   static_assert(kPlan.b_lm == 1 && NSLOT >= 2, "a K and a V slot at least");
@@ -67,10 +74,20 @@ struct FwdCfg {
   static constexpr uint32_t SLOT_BYTES = NBOX * KV_BOX_BYTES;
   static constexpr uint32_t Q_OFF = 0;
   static constexpr uint32_t RING_OFF = NQT * Q_TILE_BYTES;
-  static constexpr uint32_t STG_OFF = RING_OFF + NSLOT * SLOT_BYTES;  // O staging per tile
-  static constexpr uint32_t BAR_OFF = STG_OFF + NQT * BM * D * 2;
-  // barriers: q_full[2], q_empty[2], full[NSLOT], empty[NSLOT], s[2], p[2][2], o[2], o_empty[2], drain
-  static constexpr int NBAR = 4 + 2 * NSLOT + 11;
+  static constexpr uint32_t STG_OFF = RING_OFF + NSLOT * SLOT_BYTES;  // O staging
+  static constexpr uint32_t BAR_OFF = STG_OFF + (SHARED_STG ? 1 : NQT) * BM * D * 2;
+  // barriers: q_full[2], q_empty[2], full[NSLOT], empty[NKE], s[2], p[2][2], o[2], o_empty[2],
+  // stg_free[2][4], drain
+  // Released tiles: K number n (counted over all items) and the V before it are released
+  // together by the commit behind the last S of K number n, on barrier n % NKE.
+  static constexpr int NKE = (NSLOT + 1) / 2;
+  // The MMA warp waits for the next V before it issues tile 1's next S, while P.V keeps the
+  // tensor pipe busy, and not after it, when the pipe runs dry meanwhile: at D = 128 +2.3 % (B4
+  // H32 S2048: 184.4 -> 180.3 us); at D = 64, where the softmax bounds the step, it would
+  // hold that S back (523 -> 529 us on H64/16 S8192 causal).  A ring of two slots cannot: that
+  // V's slot is only released by this S.
+  static constexpr bool V_FIRST = D == 128 && NSLOT >= 3;
+  static constexpr int NBAR = 4 + NSLOT + NKE + 11 + 8;
   static constexpr uint32_t TMEM_PTR_OFF = BAR_OFF + NBAR * 8;
   static constexpr uint32_t ABORT_OFF = TMEM_PTR_OFF + 8;
   static constexpr uint32_t BYTES = ABORT_OFF + 16 + 1024;  // + alignment slack
@@ -254,7 +271,10 @@ __device__ __forceinline__ Item make_item_t(const FwdParams& p, const SeqCursor&
 // halves (arriving on bar_p and bar_p + 8 after each, so that P.V can start on the first
 // half), rescale O at o_tm when the max moved (after waiting for the previous P.V on
 // bar_o with parity par_o), and accumulate the row sum.  Returns false if a wait gave up.
-template <int D, int BN>
+// PV_DONE: S is only ready after the previous P.V of this tile (its MMAs are issued behind
+// it by the same thread, and a commit covers everything issued before), so the rescale
+// need not wait for bar_o.
+template <int D, int BN, bool PV_DONE = false>
 __device__ __forceinline__ bool softmax_step(uint32_t s_tm, uint32_t o_tm, uint32_t bar_s,
                                              uint32_t par_s, uint32_t bar_p, uint32_t bar_o,
                                              uint32_t par_o, bool first, int kbase, int limit,
@@ -336,7 +356,7 @@ __device__ __forceinline__ bool softmax_step(uint32_t s_tm, uint32_t o_tm, uint3
     // O must hold the previous P.V before it is rescaled, and be rescaled before this
     // tile's P.V starts (the first-half arrive below).
     if (half == 0 && !first && __any_sync(0xffffffffu, need)) {
-      if (!mbar_wait_warp(bar_o, par_o, ctl, ab)) return false;
+      if (!PV_DONE && !mbar_wait_warp(bar_o, par_o, ctl, ab)) return false;
       tc_fence_after();
       const uint64_t a2 = f2(alpha, alpha);
 #pragma unroll 1
@@ -373,12 +393,19 @@ __device__ __forceinline__ bool softmax_step(uint32_t s_tm, uint32_t o_tm, uint3
 // Ragged batches (VARLEN): O is [total_q, Hq, D] and the store box is 32 rows of one head;
 // a warp whose 32 rows run past its sequence's end writes its valid rows with plain
 // stores instead (a TMA store would spill into the next sequence), and LSE is [Hq, total_q].
+// bar_mine / bar_peer (0: the block is this warp's own): the two query tiles' warps of the
+// same rows share one staging block and take turns.  The warp waits until its peer's last
+// store has read the block (bar_peer, par_peer; peer_used: there was one), and releases the
+// block to the peer (bar_mine) once its own store has read it, a wait that falls into the
+// item boundary, where this warp waits for the next item's first S anyway.
 template <int D, bool VARLEN = false>
 __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, uint32_t par_o,
                                                  uint32_t bar_oe, float m_run, float l_run,
                                                  int row, int q_z, const FwdParams& p,
                                                  const Abort& ab, const CUtensorMap* tm_o,
-                                                 uint32_t stg, int qb = 0, int sq = 0) {
+                                                 uint32_t stg, int qb = 0, int sq = 0,
+                                                 uint32_t bar_mine = 0, uint32_t bar_peer = 0,
+                                                 uint32_t par_peer = 0, bool peer_used = false) {
   const int lane = threadIdx.x & 31;
   if (!mbar_wait_warp(bar_o, par_o, p.ctl, ab)) return false;
   tc_fence_after();
@@ -404,9 +431,11 @@ __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, 
   }
   tc_fence_before();
   mbar_arrive(bar_oe);  // O is in registers: the next item's P.V may overwrite it
+  if (peer_used && !mbar_wait_warp(bar_peer, par_peer, p.ctl, ab)) return false;
   if constexpr (VARLEN) {
     const int row0 = row - lane;  // the warp's rows are row0 .. row0 + 31
     if (row0 + 32 > sq) {
+      if (bar_mine && lane == 0) mbar_arrive(bar_mine);  // nothing of this warp is staged
       if (row < sq) {
         uint4* dst = reinterpret_cast<uint4*>(p.o + (static_cast<size_t>(qb + row) * p.Hq + q_z) * D);
 #pragma unroll
@@ -434,6 +463,10 @@ __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, 
 #pragma unroll
       for (int x = 0; x < D / 64; ++x) tma_store_3d(tm_o, stg + x * 4096u, x * 64, q_z, qb + row);
       bulk_commit_group();
+      if (bar_mine) {
+        bulk_wait_group_read0();
+        mbar_arrive(bar_mine);
+      }
     }
     if (p.lse)
       p.lse[static_cast<size_t>(q_z) * p.total_q + qb + row] = l_run > 0.f ? (m_run + log2f(l_run)) * kLn2 : -INFINITY;
@@ -443,6 +476,10 @@ __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, 
 #pragma unroll
     for (int x = 0; x < D / 64; ++x) tma_store_3d(tm_o, stg + x * 4096u, x * 64, row, q_z);
     bulk_commit_group();
+    if (bar_mine) {
+      bulk_wait_group_read0();
+      mbar_arrive(bar_mine);
+    }
   }
   if (row < p.Sq && p.lse)
     p.lse[static_cast<size_t>(q_z) * p.Sq + row] = l_run > 0.f ? (m_run + log2f(l_run)) * kLn2 : -INFINITY;
@@ -491,12 +528,13 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
   const uint32_t bar_q = sbase + C::BAR_OFF;       // [2] Q_t loaded (once per item)
   const uint32_t bar_qe = bar_q + 16;              // [2] Q_t no longer read (once per item)
   const uint32_t bar_full = bar_qe + 16;           // [NSLOT]
-  const uint32_t bar_empty = bar_full + 8 * C::NSLOT;
-  const uint32_t bar_s = bar_empty + 8 * C::NSLOT;  // [2] S_t ready
+  const uint32_t bar_empty = bar_full + 8 * C::NSLOT;  // [NKE] K number n and the V before it are no longer read
+  const uint32_t bar_s = bar_empty + 8 * C::NKE;       // [2] S_t ready
   const uint32_t bar_p = bar_s + 16;                // [2][2] half h of P_t written (h = 0: and O_t rescaled)
   const uint32_t bar_o = bar_p + 32;                // [2] P_t V_j accumulated into O_t
   const uint32_t bar_oe = bar_o + 16;               // [2] O_t read out by the epilogue
-  const uint32_t bar_drain = bar_oe + 16;
+  const uint32_t bar_stg = bar_oe + 16;             // [2][4] tile t's warp w is done with the shared staging block
+  const uint32_t bar_drain = bar_stg + 64;
   uint32_t* tmem_ptr = reinterpret_cast<uint32_t*>(smem + C::TMEM_PTR_OFF);
   Abort ab{reinterpret_cast<volatile int*>(smem + C::ABORT_OFF)};
 
@@ -505,10 +543,8 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
       mbar_init(bar_q + 8 * t, 1);
       mbar_init(bar_qe + 8 * t, 1);
     }
-    for (int s = 0; s < C::NSLOT; ++s) {
-      mbar_init(bar_full + 8 * s, 1);
-      mbar_init(bar_empty + 8 * s, 1);
-    }
+    for (int s = 0; s < C::NSLOT; ++s) mbar_init(bar_full + 8 * s, 1);
+    for (int n = 0; n < C::NKE; ++n) mbar_init(bar_empty + 8 * n, 1);
     for (int t = 0; t < 2; ++t) {
       mbar_init(bar_s + 8 * t, 1);
       mbar_init(bar_p + 16 * t, C::BM);
@@ -516,6 +552,7 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
       mbar_init(bar_o + 8 * t, 1);
       mbar_init(bar_oe + 8 * t, C::BM);
     }
+    for (int i = 0; i < 8; ++i) mbar_init(bar_stg + 8 * i, 1);
     mbar_init(bar_drain, 1);
     *ab.flag = 0;
     *(ab.flag + 1) = 0;
@@ -572,8 +609,12 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
                                                          nx.kb);
             }
           }
-          const int slot = pos % C::NSLOT, round = pos / C::NSLOT;
-          if (!(ok = mbar_wait(bar_empty + 8 * slot, (round & 1) ^ 1, p.ctl, ab))) break;
+          const int slot = pos % C::NSLOT;
+          // the slot's last tile, at position pos - NSLOT, is released with K number n
+          if (pos >= C::NSLOT) {
+            const int n = (pos - C::NSLOT + 1) >> 1;
+            if (!(ok = mbar_wait(bar_empty + 8 * (n % C::NKE), (n / C::NKE) & 1, p.ctl, ab))) break;
+          }
           issued = pos + 1;
           if (p.ctl.inject == 2 && pos == 2) {  // test hook: never load this tile
             skipped = pos;
@@ -643,12 +684,12 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
         tc_fence_after();
         issue_s(1, pos);
         tc_commit_el(bar_s + 8);
-        tc_commit_el(bar_empty + 8 * (pos % C::NSLOT));
+        tc_commit_el(bar_empty + 8 * ((pos >> 1) % C::NKE));
+        if (!(ok = wait_slot(pos + 1))) break;
         if (nt == 1) tc_commit_el(bar_qe + 8);  // every S of tile 1 issued
         for (int j = 0; j < nt; ++j) {
           const int vpos = pos + 2 * j + 1, kpos = pos + 2 * j + 2;
           const bool more = j + 1 < nt;
-          if (!(ok = wait_slot(vpos))) break;
           if (j < nt0) {  // query tile 0 stops at its own diagonal
             if (!(ok = mbar_wait_warp(bar_p, (cnt0 + j) & 1, p.ctl, ab))) break;
             // O_0 of the previous item must have been read out
@@ -658,7 +699,7 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
             if (!(ok = mbar_wait_warp(bar_p + 8, (cnt0 + j) & 1, p.ctl, ab))) break;
             tc_fence_after();
             issue_pv(0, vpos, true, 1);
-            tc_commit_el(bar_o);
+            if (j + 1 == nt0) tc_commit_el(bar_o);
           }
           if (more) {
             if (!(ok = wait_slot(kpos))) break;
@@ -676,12 +717,22 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
           if (!(ok = mbar_wait_warp(bar_p + 24, (cnt1 + j) & 1, p.ctl, ab))) break;
           tc_fence_after();
           issue_pv(1, vpos, true, 1);
-          tc_commit_el(bar_o + 8);
-          tc_commit_el(bar_empty + 8 * (vpos % C::NSLOT));
-          if (more) {
+          // Few commits: each takes a place in the short queue of issued MMAs, and with it some
+          // of the time that the warp has for its next waits before the pipe runs dry.  The
+          // rescale needs none (S follows P.V), O is only awaited at the item's end, and V_j is
+          // released with K_{j+1}.
+          if (!more) {
+            tc_commit_el(bar_o + 8);
+          } else {
+            if constexpr (C::V_FIRST) {
+              if (!(ok = wait_slot(vpos + 2))) break;
+            }
             issue_s(1, kpos);
             tc_commit_el(bar_s + 8);
-            tc_commit_el(bar_empty + 8 * (kpos % C::NSLOT));
+            tc_commit_el(bar_empty + 8 * ((kpos >> 1) % C::NKE));
+            if constexpr (!C::V_FIRST) {
+              if (!(ok = wait_slot(vpos + 2))) break;
+            }
             if (j + 2 == nt) tc_commit_el(bar_qe + 8);  // tile 1's last S of the item
           }
         }
@@ -703,7 +754,11 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     const uint32_t o_tm = tmem + lane_addr + C::O_COL + t * D;
     const uint32_t my_bar_s = bar_s + 8 * t, my_bar_p = bar_p + 16 * t, my_bar_o = bar_o + 8 * t;
     const uint32_t my_bar_oe = bar_oe + 8 * t;
-    const uint32_t stg_q = sbase + C::STG_OFF + static_cast<uint32_t>(warp) * (32 * D * 2);
+    const uint32_t stg_q =
+        sbase + C::STG_OFF + static_cast<uint32_t>(C::SHARED_STG ? warp & 3 : warp) * (32 * D * 2);
+    // shared staging: tile 0's warp goes first, tile 1's after it, item by item
+    const uint32_t bar_mine = C::SHARED_STG ? bar_stg + 32 * t + 8 * (warp & 3) : 0;
+    const uint32_t bar_peer = C::SHARED_STG ? bar_stg + 32 * (t ^ 1) + 8 * (warp & 3) : 0;
     const float c = p.c;
     const uint64_t c2 = f2(c, c);
     const int off = p.Skv - p.Sq;
@@ -720,14 +775,15 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
       const int my_tiles = t == 0 ? it.n_tiles0 : it.n_tiles;
       float m_run = -INFINITY, l_run = 0.f;
       for (int j = 0; ok && j < my_tiles; ++j)
-        ok = softmax_step<D, C::BN>(s_tm, o_tm, my_bar_s, (cnt + j) & 1, my_bar_p, my_bar_o,
+        ok = softmax_step<D, C::BN, true>(s_tm, o_tm, my_bar_s, (cnt + j) & 1, my_bar_p, my_bar_o,
                                     (cnt + j - 1) & 1, j == 0, j * C::BN, limit, c, c2, m_run,
                                     l_run, p.ctl, ab);
       if (!ok) break;
       // epilogue: hand O_t back to the MMA warp, O / l -> bf16 rows, LSE
-      if (!(ok = softmax_epilogue<D, VARLEN>(o_tm, my_bar_o, (cnt + my_tiles - 1) & 1, my_bar_oe, m_run,
+      if (!(ok = softmax_epilogue<D, VARLEN>(o_tm, my_bar_o, r & 1, my_bar_oe, m_run,
                                              l_run, row, it.q_z, p, ab, &tm_o, stg_q,
-                                             VARLEN ? it.qb : 0, VARLEN ? it.sq : 0)))
+                                             VARLEN ? it.qb : 0, VARLEN ? it.sq : 0, bar_mine, bar_peer,
+                                             t == 1 ? r & 1 : (r - 1) & 1, C::SHARED_STG && (t == 1 || r > 0))))
         break;
       cnt += my_tiles;
     }
@@ -1765,7 +1821,7 @@ cudaError_t launch_fwd_d(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t st
   static PerDeviceOnce configured1, configured2, configured3;
   constexpr int kModelDesign = model::fwd_plan(D).design;
   const int design = a.design ? a.design : kModelDesign;
-  if (design == 2 && a.slots > 0 && a.slots != FwdCfg<D>::NSLOT) {
+  if (design == 2 && a.slots > 0 && a.slots != FwdCfg<D>::kPlan.kv_slots) {
     bool handled = false;
     const cudaError_t e = launch_two_tile_slots<D>(a, ctl, stream, &handled);
     if (handled) return e;
