@@ -27,6 +27,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -87,7 +88,8 @@ struct FwdCfg {
   // hold that S back (523 -> 529 us on H64/16 S8192 causal).  A ring of two slots cannot: that
   // V's slot is only released by this S.
   static constexpr bool V_FIRST = D == 128 && NSLOT >= 3;
-  static constexpr int NBAR = 4 + NSLOT + NKE + 11 + 8;
+  // ... and of a cluster that shares items: done, xdone, rdy[8], xf[8]
+  static constexpr int NBAR = 4 + NSLOT + NKE + 11 + 8 + 18;
   static constexpr uint32_t TMEM_PTR_OFF = BAR_OFF + NBAR * 8;
   static constexpr uint32_t ABORT_OFF = TMEM_PTR_OFF + 8;
   static constexpr uint32_t BYTES = ABORT_OFF + 16 + 1024;  // + alignment slack
@@ -96,6 +98,9 @@ struct FwdCfg {
   static constexpr uint32_t O_COL = 2 * BN;   // + t * D
   static_assert(BYTES <= 227 * 1024, "shared memory budget");
   static_assert(O_COL + NQT * D <= TMEM_COLS, "TMEM budget");
+  // a cluster's partials of one item: S - 1 sources of D / S fp32 columns and (m, l) per row
+  static_assert(SLOTS != 0 || 7 * (D / 8 * 4 + 8) * 256 <= RING_OFF + (NSLOT + 1) / 2 * SLOT_BYTES,
+                "partials fit in the Q tiles and the K slots");
 };
 
 struct FwdParams {
@@ -113,22 +118,30 @@ struct FwdParams {
   const int32_t* cu_q;  // [B + 1] first query token of each sequence
   const int32_t* cu_k;  // [B + 1] first key token of each sequence
   int B, total_q;       // sequences; query tokens (the row stride of LSE [Hq, total_q])
+  // two-tile design, dense: a plane's rows are the rows of 2^pack_log2 query heads of one
+  // kv head (row i of the plane: query i >> pack_log2 of head i mod 2^pack_log2)
+  int pack_log2, planes_per_kv, q_rows;
 };
 
-// One work item of a persistent CTA: a pair of 128-row query tiles of one (b, h).
+// One work item of a persistent CTA: a pair of 128-row query tiles of one (b, h), or of one
+// plane of packed heads.
 struct Item {
   int b, h, q_z, kv_z, q0, n_tiles0, n_tiles;
   int sq, skv, qb, kb;  // ragged batches: the sequence's lengths and first tokens
+  int q1;   // two-tile design: tile 1's first row (tile 0's is q0; n_tiles0 = 0: no tile 0)
+  int kt0;  // first KV tile of this CTA's share of the item (0 unless a cluster splits it)
 };
 
 // The r-th item of this CTA (-1 once it has none left).  Causal items are ordered
 // heaviest first (within blocks of planes, see item_coords) and dealt out in a snake
 // order (CTA c takes item c of even rounds and item G-1-c of odd rounds) so that long and
 // short items even out per CTA.
-__device__ __forceinline__ int item_index(const FwdParams& p, int r) {
-  const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x);
+__device__ __forceinline__ int item_index(const FwdParams& p, int r, int c, int G) {
   const long long idx = static_cast<long long>(r) * G + ((p.causal && (r & 1)) ? G - 1 - c : c);
   return idx < p.n_items ? static_cast<int>(idx) : -1;
+}
+__device__ __forceinline__ int item_index(const FwdParams& p, int r) {
+  return item_index(p, r, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x));
 }
 
 // Item idx -> (position pos of its query tile or tile pair within the plane, plane bh).
@@ -208,12 +221,11 @@ __device__ __forceinline__ SeqCursor seq_cursor(const FwdParams& p) {
 // Dense: the r-th item's index (see item_index).  Ragged: the same dealing over the
 // unbounded index space, with the cursor moved to the item's sequence; -1 past the last.
 template <int ROWS, bool VARLEN>
-__device__ __forceinline__ int item_index_t(const FwdParams& p, int r, SeqCursor& cur) {
+__device__ __forceinline__ int item_index_t(const FwdParams& p, int r, SeqCursor& cur, int c, int G) {
   if constexpr (!VARLEN) {
     (void)cur;
-    return item_index(p, r);
+    return item_index(p, r, c, G);
   } else {
-    const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x);
     const long long idx = static_cast<long long>(r) * G + ((p.causal && (r & 1)) ? G - 1 - c : c);
     while (cur.b < p.B && idx >= cur.first + static_cast<long long>(cur.pairs) * p.Hq) {
       cur.first += static_cast<long long>(cur.pairs) * p.Hq;
@@ -227,12 +239,33 @@ __device__ __forceinline__ int item_index_t(const FwdParams& p, int r, SeqCursor
 // Ragged item: causal takes a sequence's heaviest pairs (last rows) first over all heads;
 // non-causal takes one head's pairs in a row (they share its K/V in L2).  At least one KV
 // tile is processed even when no key is visible (fully masked: O = 0, LSE = -inf).
-template <int D, bool VARLEN>
+// Dense item: query tiles of a plane of packed heads.  An item whose second tile would lie
+// past the plane's rows keeps its one tile as tile 1 (which walks the whole item) and has no
+// tile 0.
+template <int D, bool VARLEN, bool ONE = true>
 __device__ __forceinline__ Item make_item_t(const FwdParams& p, const SeqCursor& cur, int idx) {
   using C = FwdCfg<D>;
   if constexpr (!VARLEN) {
     (void)cur;
-    return make_item<D>(p, idx);
+    int pos, z;
+    item_coords(p, idx, pos, z);
+    Item it;
+    it.b = it.h = it.sq = it.skv = it.qb = it.kb = 0;
+    it.q_z = z;
+    it.kv_z = z / p.planes_per_kv;
+    it.q0 = pos * (C::NQT * C::BM);
+    const bool two = !ONE || it.q0 + C::BM < p.q_rows;
+    it.q1 = two ? it.q0 + C::BM : it.q0;
+    int n_kv0 = p.Skv, n_kv1 = p.Skv;
+    if (p.causal) {
+      const int off = p.Skv - p.Sq;  // bottom-right causal offset
+      n_kv0 = min(p.Skv, ((it.q0 + C::BM) >> p.pack_log2) + off);
+      n_kv1 = min(p.Skv, ((it.q1 + C::BM) >> p.pack_log2) + off);
+    }
+    it.n_tiles0 = two ? (n_kv0 + C::BN - 1) / C::BN : 0;
+    it.n_tiles = (n_kv1 + C::BN - 1) / C::BN;
+    it.kt0 = 0;
+    return it;
   } else {
     const int in = static_cast<int>(idx - cur.first);
     int pos, h;
@@ -253,16 +286,28 @@ __device__ __forceinline__ Item make_item_t(const FwdParams& p, const SeqCursor&
     it.kb = p.cu_k[cur.b];
     it.skv = p.cu_k[cur.b + 1] - it.kb;
     it.q0 = pos * (C::NQT * C::BM);
+    const bool two = it.q0 + C::BM < it.sq;
+    it.q1 = two ? it.q0 + C::BM : it.q0;
     const int off = it.skv - it.sq;
     int n_kv0 = it.skv, n_kv1 = it.skv;
     if (p.causal) {
       n_kv0 = min(it.skv, it.q0 + C::BM + off);
-      n_kv1 = min(it.skv, it.q0 + 2 * C::BM + off);
+      n_kv1 = min(it.skv, it.q1 + C::BM + off);
     }
-    it.n_tiles0 = max(1, (n_kv0 + C::BN - 1) / C::BN);
-    it.n_tiles = max(it.n_tiles0, (n_kv1 + C::BN - 1) / C::BN);
+    it.n_tiles0 = two ? max(1, (n_kv0 + C::BN - 1) / C::BN) : 0;
+    it.n_tiles = max(1, max(it.n_tiles0, (n_kv1 + C::BN - 1) / C::BN));
+    it.kt0 = 0;
     return it;
   }
+}
+
+// The share of an item's KV tiles that CTA `rank` of a cluster of S takes: tiles
+// [n rank / S, n (rank + 1) / S).  n_tiles and n_tiles0 become this CTA's own counts.
+__device__ __forceinline__ void split_item(Item& it, int rank, int S) {
+  const int lo = it.n_tiles * rank / S, hi = it.n_tiles * (rank + 1) / S;
+  it.kt0 = lo;
+  it.n_tiles = hi - lo;
+  it.n_tiles0 = max(0, min(it.n_tiles0 - lo, hi - lo));
 }
 
 // One online-softmax step of one query row (this thread's TMEM lane) over a BN-key
@@ -398,7 +443,13 @@ __device__ __forceinline__ bool softmax_step(uint32_t s_tm, uint32_t o_tm, uint3
 // store has read the block (bar_peer, par_peer; peer_used: there was one), and releases the
 // block to the peer (bar_mine) once its own store has read it, a wait that falls into the
 // item boundary, where this warp waits for the next item's first S anyway.
-template <int D, bool VARLEN = false>
+// PACKED: O rows are rows of a plane of packed heads (FwdParams::pack_log2; the 32 rows of
+// a warp are one box of the 4-D output map).
+__device__ __forceinline__ size_t packed_lse_row(const FwdParams& p, int q_z, int row) {
+  return ((static_cast<size_t>(q_z) << p.pack_log2) + (row & ((1 << p.pack_log2) - 1))) * p.Sq + (row >> p.pack_log2);
+}
+
+template <int D, bool VARLEN = false, bool PACKED = false>
 __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, uint32_t par_o,
                                                  uint32_t bar_oe, float m_run, float l_run,
                                                  int row, int q_z, const FwdParams& p,
@@ -474,12 +525,21 @@ __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, 
   }
   if (lane == 0) {
 #pragma unroll
-    for (int x = 0; x < D / 64; ++x) tma_store_3d(tm_o, stg + x * 4096u, x * 64, row, q_z);
+    for (int x = 0; x < D / 64; ++x) {
+      if constexpr (PACKED)
+        tma_store_4d(tm_o, stg + x * 4096u, x * 64, 0, row >> p.pack_log2, q_z);
+      else
+        tma_store_3d(tm_o, stg + x * 4096u, x * 64, row, q_z);
+    }
     bulk_commit_group();
     if (bar_mine) {
       bulk_wait_group_read0();
       mbar_arrive(bar_mine);
     }
+  }
+  if constexpr (PACKED) {
+    if (row < p.q_rows && p.lse) p.lse[packed_lse_row(p, q_z, row)] = l_run > 0.f ? (m_run + log2f(l_run)) * kLn2 : -INFINITY;
+    return true;
   }
   if (row < p.Sq && p.lse)
     p.lse[static_cast<size_t>(q_z) * p.Sq + row] = l_run > 0.f ? (m_run + log2f(l_run)) * kLn2 : -INFINITY;
@@ -488,13 +548,18 @@ __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, 
 
 // Bring the next work item's query tiles and first K/V tiles into L2 while the current
 // item still runs, so that its start waits on an L2 hit rather than HBM.
-template <int D, int NQT, int BM, bool VARLEN = false>
+template <int D, int NQT, int BM, bool VARLEN = false, bool PACKED = false>
 __device__ __forceinline__ void prefetch_item_l2(const CUtensorMap* tm_q, const CUtensorMap* tm_k,
                                                  const CUtensorMap* tm_v, int q0, int q_z, int kv_z,
-                                                 int qb = 0, int kb = 0) {
+                                                 int qb = 0, int kb = 0, int pack_log2 = 0) {
 #pragma unroll
   for (int x = 0; x < D / 64; ++x) {
-    if constexpr (VARLEN) {
+    if constexpr (PACKED) {
+#pragma unroll
+      for (int t = 0; t < NQT; ++t) tma_prefetch_l2_4d(tm_q, x * 64, 0, (q0 + t * BM) >> pack_log2, q_z);
+      tma_prefetch_l2_3d(tm_k, x * 64, kb, kv_z);
+      tma_prefetch_l2_3d(tm_v, x * 64, kb, kv_z);
+    } else if constexpr (VARLEN) {
 #pragma unroll
       for (int t = 0; t < NQT; ++t) tma_prefetch_l2_3d(tm_q, x * 64, q_z, qb + q0 + t * BM);
       tma_prefetch_l2_3d(tm_k, x * 64, kv_z, kb);
@@ -508,10 +573,184 @@ __device__ __forceinline__ void prefetch_item_l2(const CUtensorMap* tm_q, const 
   }
 }
 
+// Epilogue of one query row when a cluster of S CTAs shares the item.  Each CTA holds the
+// row's (m, l) and unnormalised O over its own KV tiles; CTA q of the cluster finishes
+// columns [q D / S, (q + 1) D / S) of both query tiles.  So the warp sends, for every other
+// CTA, its rows' (m, l) and those columns of O (fp32) into that CTA's Q tiles and K slots
+// (the even ring slots) -- idle once that CTA's last S of the item is done, which it
+// announces on bar_rdy[its rank] a tile-step before it needs the partials -- waits for
+// the S - 1 partials of its own rows (bar_xf[warp]), and sums the S partials in rank order
+// (the result does not depend on timing), O = sum 2^(m_s - M) O_s / sum 2^(m_s - M) l_s.
+// Layout (of the 16-byte units, see partial_at), per source CTA: float4 chunk c of row r at (c * 256 + r) * 16 (a
+// warp's 32 rows are contiguous: no bank conflicts on either side), then (m, l) per row.
+// has_tiles: this CTA walked KV tiles of the row's tile; active: the item has that tile.
+// The finished columns go through the warp's staging block (4 KB) so that a warp stores
+// whole rows' pieces: stored straight from the row threads, 32 rows per instruction, the
+// stores alone took 2 us of the exchange's 7.  Not inlined: its registers would spill
+// values of the softmax loop around it.
+// Byte `off` of the partials' space: the Q tiles and ring slot 0, which follow one another,
+// then ring slots 2, 4, ...
+template <class C>
+__device__ __forceinline__ uint32_t partial_at(uint32_t sbase, uint32_t off) {
+  constexpr uint32_t kHead = C::RING_OFF - C::Q_OFF + C::SLOT_BYTES;
+  static_assert(C::NSLOT % 2 == 0, "K tiles sit in the even ring slots");
+  const uint32_t skip = off < kHead ? 0u : ((off - kHead) / C::SLOT_BYTES + 1) * C::SLOT_BYTES;
+  return sbase + C::Q_OFF + off + skip;
+}
+
+struct SplitRow {
+  __nv_bfloat16* o;
+  float* lse;
+  int Sq, q_rows, pack_log2;
+  int row, q_z;         // this thread's packed row of plane q_z
+  float m, l;           // this CTA's running max and sum
+  bool has_tiles, active, first;
+  uint32_t par_o, par_x, par_f;  // phases: this tile's O, the item, the items that had this tile
+};
+struct SplitBars {
+  uint32_t o, oe, rdy, xf, xdone;
+};
+template <int D, int S>
+__device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars bar, uint32_t o_tm, uint32_t sbase,
+                                            uint32_t stg, int warp, int rank, const KernelCtl ctl, const Abort ab) {
+  constexpr int kRows = 256;
+  constexpr int W = D / S;                              // columns this CTA finishes
+  constexpr uint32_t kO = W * 4 * kRows, kSrc = kO + 8 * kRows;  // one source's O, all of its partials
+  using C = FwdCfg<D>;
+  constexpr int U = 8;  // columns finished at a time (more of them spill)
+  static_assert(W % 8 == 0, "whole 16-byte stores of bf16");
+  const int lane = threadIdx.x & 31;
+  const int rb = warp * 32 + lane;
+  if (r.active && r.has_tiles) {
+    if (!mbar_wait_warp(bar.o, r.par_o, ctl, ab)) return false;
+    tc_fence_after();
+  }
+  // (also without a tile: no warp may run an item ahead of these barriers' phases)
+  if (!r.active && !r.first && !mbar_wait_warp(bar.xdone, r.par_x ^ 1, ctl, ab)) return false;
+#pragma unroll
+  for (int q = 0; q < S; ++q)
+    if (q != rank && !mbar_wait_cluster_warp(bar.rdy + 8 * q, r.par_x, ctl, ab)) return false;
+  if (r.active) {
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+      const uint32_t mine = static_cast<uint32_t>(rank < q ? rank : rank - (rank > q)) * kSrc;  // my place in CTA q
+      if (q != rank) st_dsmem_f2(map_shared_rank(partial_at<C>(sbase, mine + kO + rb * 8), q), r.m, r.l);
+    }
+    if (r.has_tiles) {
+#pragma unroll
+      for (int ch = 0; ch < D / 32; ++ch) {
+        uint32_t rr[32];
+        tmem_ld32(o_tm + ch * 32, rr);
+        tmem_wait_ld();
+        reg_fence32(rr);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int col = ch * 32 + u * 4;
+          const int q = col / W;
+          const uint32_t mine = static_cast<uint32_t>(rank < q ? rank : rank - (rank > q)) * kSrc;
+          if (q != rank)
+            st_dsmem_v4(map_shared_rank(partial_at<C>(sbase, mine + (col - q * W) / 4 * kRows * 16 + rb * 16), q),
+                        rr[4 * u], rr[4 * u + 1], rr[4 * u + 2], rr[4 * u + 3]);
+        }
+      }
+    }
+    fence_acq_rel_cluster();
+    __syncwarp();
+    if (lane < S && lane != rank) mbar_arrive_cluster(map_shared_rank(bar.xf + 8 * warp, lane));
+    if (!mbar_wait_cluster_warp(bar.xf + 8 * warp, r.par_f, ctl, ab)) return false;
+    // the S partials' weights, in rank order
+    float w[S], l = 0.f, M = r.m;
+    float2 ml[S];
+    uint32_t src[S];  // source s's place
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      src[s] = static_cast<uint32_t>(s < rank ? s : s - (s > rank)) * kSrc;
+      ml[s] = s == rank ? make_float2(r.m, r.l) : ld_shared_f2(partial_at<C>(sbase, src[s] + kO + rb * 8));
+      M = fmaxf(M, ml[s].x);
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      w[s] = ml[s].x == -INFINITY ? 0.f : ex2(ml[s].x - M);  // 0: that CTA saw no key of the row
+      l = fmaf(w[s], ml[s].y, l);
+    }
+    const float inv_l = l > 0.f ? 1.f / l : 0.f;
+    constexpr int kChunks = W / 8;  // 16-byte chunks of a staged row, swizzled over the banks
+    const uint32_t my_row = stg + static_cast<uint32_t>(lane) * (W * 2);
+    const int swz = lane / (8 / kChunks) & (kChunks - 1);
+#pragma unroll 1
+    for (int c = 0; c < W; c += U) {
+      uint32_t own[U];
+      if (r.has_tiles) {
+#pragma unroll
+        for (int i = 0; i < U; i += 8) tmem_ld8(o_tm + rank * W + c + i, own + i);
+      }
+      float acc[U];
+#pragma unroll
+      for (int i = 0; i < U; ++i) acc[i] = 0.f;
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        if (s == rank) {
+          if (r.has_tiles) {
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < U; i += 8) reg_fence8(own + i);
+#pragma unroll
+            for (int i = 0; i < U; ++i) acc[i] = fmaf(w[s], __uint_as_float(own[i]), acc[i]);
+          }
+        } else if (w[s] != 0.f) {  // (a CTA without tiles of this row has sent no O)
+          uint4 v[U / 4];
+#pragma unroll
+          for (int i = 0; i < U / 4; ++i) 
+            v[i] = ld_shared_v4(partial_at<C>(sbase, src[s] + static_cast<uint32_t>((c / 4 + i) * kRows * 16 + rb * 16)));
+#pragma unroll
+          for (int i = 0; i < U / 4; ++i) {
+            acc[4 * i] = fmaf(w[s], __uint_as_float(v[i].x), acc[4 * i]);
+            acc[4 * i + 1] = fmaf(w[s], __uint_as_float(v[i].y), acc[4 * i + 1]);
+            acc[4 * i + 2] = fmaf(w[s], __uint_as_float(v[i].z), acc[4 * i + 2]);
+            acc[4 * i + 3] = fmaf(w[s], __uint_as_float(v[i].w), acc[4 * i + 3]);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < U; i += 8)
+        st_shared_v4(my_row + static_cast<uint32_t>(((c + i) / 8 ^ swz) << 4),
+                     pack_bf16x2(acc[i] * inv_l, acc[i + 1] * inv_l), pack_bf16x2(acc[i + 2] * inv_l, acc[i + 3] * inv_l),
+                     pack_bf16x2(acc[i + 4] * inv_l, acc[i + 5] * inv_l),
+                     pack_bf16x2(acc[i + 6] * inv_l, acc[i + 7] * inv_l));
+    }
+    if (r.has_tiles) {
+      tc_fence_before();
+      mbar_arrive(bar.oe);
+    }
+    const int mask = (1 << r.pack_log2) - 1;
+    const size_t head0 = static_cast<size_t>(r.q_z) << r.pack_log2;
+    if (rank == 0 && r.row < r.q_rows && r.lse)
+      r.lse[(head0 + (r.row & mask)) * r.Sq + (r.row >> r.pack_log2)] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < kChunks; ++k) {
+      const int i = k * 32 + lane, rr = i / kChunks, j = i % kChunks;
+      const int row = r.row - lane + rr;
+      const uint4 v = ld_shared_v4(stg + static_cast<uint32_t>(rr * (W * 2)) +
+                                   static_cast<uint32_t>((j ^ (rr / (8 / kChunks) & (kChunks - 1))) << 4));
+      if (row < r.q_rows)
+        reinterpret_cast<uint4*>(r.o + ((head0 + (row & mask)) * r.Sq + (row >> r.pack_log2)) * D + rank * W)[j] = v;
+    }
+  }
+  fence_proxy_async_smem();  // the ring's next writes are TMA loads
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar.xdone);
+  return true;
+}
+
 // VARLEN: a ragged batch packed [total, H, D]: the tensor maps are [total, H, D] views
 // (coordinates: column, head, token) and items come from the sequence cursor.  SLOTS: the
 // ring depth (0: the model's).
-template <int D, bool VARLEN = false, int SLOTS = 0>
+// SPLIT = S > 0: a cluster of S CTAs (2, 4 or 8) shares every item, each CTA walking 1/S of its KV
+// tiles, and the partial results meet over distributed shared memory (split_epilogue).
+// ONE: items of one query tile may occur (the last of a plane); without them the roles need
+// no counts of their own per tile, worth 2 % on B4 H32 S2048 (169 against 173 us).
+template <int D, bool VARLEN = false, int SLOTS = 0, int SPLIT = 0, bool ONE = true>
 __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
@@ -536,7 +775,19 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
   const uint32_t bar_stg = bar_oe + 16;             // [2][4] tile t's warp w is done with the shared staging block
   const uint32_t bar_drain = bar_stg + 64;
   uint32_t* tmem_ptr = reinterpret_cast<uint32_t*>(smem + C::TMEM_PTR_OFF);
+  const uint32_t bar_done = bar_drain + 8;          // SPLIT: every S of the item is done
+  const uint32_t bar_xdone = bar_done + 8;          // SPLIT: every warp has read the item's partials here
+  const uint32_t bar_rdy = bar_xdone + 8;           // SPLIT: [8] CTA q takes this CTA's partials
+  const uint32_t bar_xf = bar_rdy + 64;             // SPLIT: [8] the partials of warp w's rows have arrived
   Abort ab{reinterpret_cast<volatile int*>(smem + C::ABORT_OFF)};
+  constexpr int S = SPLIT ? SPLIT : 1;
+  const int rank = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+  const int wk = static_cast<int>(blockIdx.x) / S, n_wk = static_cast<int>(gridDim.x) / S;  // this worker, workers
+  auto item_of = [&](const SeqCursor& cur, int idx) {
+    Item it = make_item_t<D, VARLEN, ONE>(p, cur, idx);
+    if constexpr (SPLIT > 0) split_item(it, rank, S);
+    return it;
+  };
 
   if (threadIdx.x == 0) {
     for (int t = 0; t < 2; ++t) {
@@ -554,6 +805,14 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     }
     for (int i = 0; i < 8; ++i) mbar_init(bar_stg + 8 * i, 1);
     mbar_init(bar_drain, 1);
+    if constexpr (SPLIT > 0) {
+      mbar_init(bar_done, 1);
+      mbar_init(bar_xdone, 8);
+      for (int i = 0; i < 8; ++i) {
+        mbar_init(bar_rdy + 8 * i, 1);
+        mbar_init(bar_xf + 8 * i, S - 1);
+      }
+    }
     *ab.flag = 0;
     *(ab.flag + 1) = 0;
     fence_barrier_init();
@@ -563,6 +822,7 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_ptr;
+  if constexpr (SPLIT > 0) cluster_sync_all();  // every CTA's barriers exist before a peer arrives on them
   // Launched as a programmatic dependent of the previous kernel in the stream: the set-up
   // above touches no global memory; from here on the previous kernel's writes must be
   // complete and visible.  The next launch may then start its own set-up on SMs this
@@ -579,34 +839,42 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
       prefetch_tensormap(&tm_q);
       prefetch_tensormap(&tm_k);
       prefetch_tensormap(&tm_v);
-      int pos = 0, issued = 0, skipped = -1, q_issued[2] = {0, 0};
+      int pos = 0, issued = 0, skipped = -1, q_issued[2] = {0, 0};  // q_issued: items that had a tile t
       bool ok = true;
       SeqCursor cur = VARLEN ? seq_cursor<kRows>(p) : SeqCursor{0, 0, 0};
-      // Q_t of item r, once the previous item's S MMAs of tile t are done with its buffer
-      auto load_q = [&](int t, int r, const Item& it) -> bool {
-        if (r > 0 && !mbar_wait(bar_qe + 8 * t, (r - 1) & 1, p.ctl, ab)) return false;
+      // Q_t of the item, once the S MMAs of the tile t before it are done with its buffer
+      auto load_q = [&](int t, const Item& it) -> bool {
+        const int n = q_issued[t];
+        if (n > 0 && !mbar_wait(bar_qe + 8 * t, (n - 1) & 1, p.ctl, ab)) return false;
         mbar_expect_tx(bar_q + 8 * t, C::Q_TILE_BYTES);
-        const int qy = VARLEN ? it.q_z : it.q0 + t * C::BM;
-        const int qz = VARLEN ? it.qb + it.q0 + t * C::BM : it.q_z;
-        for (int x = 0; x < C::NBOX; ++x)
-          tma_load_3d(sbase + C::Q_OFF + t * C::Q_TILE_BYTES + x * C::Q_BOX_BYTES, &tm_q, x * C::BOX_COLS,
-                      qy, qz, bar_q + 8 * t);
-        q_issued[t] = r + 1;
+        const int row = t == 0 ? it.q0 : it.q1;
+        for (int x = 0; x < C::NBOX; ++x) {
+          const uint32_t dst = sbase + C::Q_OFF + t * C::Q_TILE_BYTES + x * C::Q_BOX_BYTES;
+          if constexpr (VARLEN)
+            tma_load_3d(dst, &tm_q, x * C::BOX_COLS, it.q_z, it.qb + row, bar_q + 8 * t);
+          else
+            tma_load_4d(dst, &tm_q, x * C::BOX_COLS, 0, row >> p.pack_log2, it.q_z, bar_q + 8 * t);
+        }
+        q_issued[t] = n + 1;
         return true;
       };
-      for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur)) >= 0; ++r) {
-        const Item it = make_item_t<D, VARLEN>(p, cur, idx);
+      for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur, wk, n_wk)) >= 0; ++r) {
+        const Item it = item_of(cur, idx);
+        // Q tiles and K slots hold the previous item's partials until every warp has read them
+        if (SPLIT && r > 0 && !(ok = mbar_wait(bar_xdone, (r - 1) & 1, p.ctl, ab))) break;
+        if (SPLIT && it.n_tiles == 0) continue;
         // Q_0 first: tile 0 finishes its S MMAs of the previous item before tile 1 does
-        if (!(ok = load_q(0, r, it))) break;
+        const bool two = !ONE || it.n_tiles0 > 0;
+        if (!(ok = load_q(two ? 0 : 1, it))) break;
         for (int jj = 0; jj < 2 * it.n_tiles; ++jj, ++pos) {  // K_0, [Q_1], V_0, K_1, V_1, ...
-          if (jj == 1 && !(ok = load_q(1, r, it))) break;
+          if (jj == 1 && two && !(ok = load_q(1, it))) break;
           if (jj == max(0, 2 * it.n_tiles - 6)) {  // three KV tiles before the end
             SeqCursor nc = cur;
-            const int nidx = item_index_t<kRows, VARLEN>(p, r + 1, nc);
+            const int nidx = item_index_t<kRows, VARLEN>(p, r + 1, nc, wk, n_wk);
             if (nidx >= 0) {
-              const Item nx = make_item_t<D, VARLEN>(p, nc, nidx);
-              prefetch_item_l2<D, C::NQT, C::BM, VARLEN>(&tm_q, &tm_k, &tm_v, nx.q0, nx.q_z, nx.kv_z, nx.qb,
-                                                         nx.kb);
+              const Item nx = item_of(nc, nidx);
+              prefetch_item_l2<D, C::NQT, C::BM, VARLEN, !VARLEN>(&tm_q, &tm_k, &tm_v, nx.q0, nx.q_z, nx.kv_z, nx.qb,
+                                                                  VARLEN ? nx.kb : nx.kt0 * C::BN, p.pack_log2);
             }
           }
           const int slot = pos % C::NSLOT;
@@ -621,7 +889,7 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
             continue;
           }
           const CUtensorMap* map = (jj & 1) ? &tm_v : &tm_k;
-          const int row = (jj >> 1) * C::BN;
+          const int row = (it.kt0 + (jj >> 1)) * C::BN;
           const int ky = VARLEN ? it.kv_z : row, kz = VARLEN ? it.kb + row : it.kv_z;
           mbar_expect_tx(bar_full + 8 * slot, C::SLOT_BYTES);
           for (int x = 0; x < C::NBOX; ++x)
@@ -670,30 +938,44 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
                    acc ? 1u : 0u);
       };
       int pos = 0, cnt0 = 0, cnt1 = 0;  // ring position of K_0; S/P/O uses so far per tile
+      int n0 = 0, n1 = 0;               // items so far that had a tile 0, a tile 1
       bool ok = true;
       SeqCursor cur = VARLEN ? seq_cursor<kRows>(p) : SeqCursor{0, 0, 0};
-      for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur)) >= 0; ++r) {
-        const Item it = make_item_t<D, VARLEN>(p, cur, idx);
+      for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur, wk, n_wk)) >= 0; ++r) {
+        const Item it = item_of(cur, idx);
         const int nt0 = it.n_tiles0, nt = it.n_tiles;
-        if (!(ok = mbar_wait_warp(bar_q, r & 1, p.ctl, ab) && wait_slot(pos))) break;
-        tc_fence_after();
-        issue_s(0, pos);
-        tc_commit_el(bar_s);
-        if (nt0 == 1) tc_commit_el(bar_qe);  // every S of tile 0 issued
-        if (!(ok = mbar_wait_warp(bar_q + 8, r & 1, p.ctl, ab))) break;
+        if (SPLIT && nt == 0) {  // nothing of this item falls to this CTA: it takes partials at once
+          if (r > 0 && !(ok = mbar_wait_warp(bar_xdone, (r - 1) & 1, p.ctl, ab))) break;
+          if (lane < S && lane != rank) mbar_arrive_cluster(map_shared_rank(bar_rdy + 8 * rank, lane));
+          continue;
+        }
+        if (!ONE || nt0 > 0) {
+          if (!(ok = mbar_wait_warp(bar_q, n0 & 1, p.ctl, ab) && wait_slot(pos))) break;
+          tc_fence_after();
+          issue_s(0, pos);
+          tc_commit_el(bar_s);
+          if (nt0 == 1) tc_commit_el(bar_qe);  // every S of tile 0 issued
+        }
+        if (!(ok = mbar_wait_warp(bar_q + 8, n1 & 1, p.ctl, ab) && (!ONE || nt0 > 0 || wait_slot(pos)))) break;
         tc_fence_after();
         issue_s(1, pos);
         tc_commit_el(bar_s + 8);
         tc_commit_el(bar_empty + 8 * ((pos >> 1) % C::NKE));
         if (!(ok = wait_slot(pos + 1))) break;
         if (nt == 1) tc_commit_el(bar_qe + 8);  // every S of tile 1 issued
+        if (SPLIT && nt == 1) tc_commit_el(bar_done);
         for (int j = 0; j < nt; ++j) {
           const int vpos = pos + 2 * j + 1, kpos = pos + 2 * j + 2;
           const bool more = j + 1 < nt;
+          if (SPLIT && !more) {  // every S is done: the peers may write their partials over Q and K
+            if (!(ok = mbar_wait_warp(bar_done, n1 & 1, p.ctl, ab))) break;
+            if (lane < S && lane != rank) mbar_arrive_cluster(map_shared_rank(bar_rdy + 8 * rank, lane));
+            __syncwarp();
+          }
           if (j < nt0) {  // query tile 0 stops at its own diagonal
             if (!(ok = mbar_wait_warp(bar_p, (cnt0 + j) & 1, p.ctl, ab))) break;
             // O_0 of the previous item must have been read out
-            if (j == 0 && r > 0 && !(ok = mbar_wait_warp(bar_oe, (r - 1) & 1, p.ctl, ab))) break;
+            if (j == 0 && n0 > 0 && !(ok = mbar_wait_warp(bar_oe, (n0 - 1) & 1, p.ctl, ab))) break;
             tc_fence_after();
             issue_pv(0, vpos, j > 0, 0);
             if (!(ok = mbar_wait_warp(bar_p + 8, (cnt0 + j) & 1, p.ctl, ab))) break;
@@ -711,7 +993,7 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
             }
           }
           if (!(ok = mbar_wait_warp(bar_p + 16, (cnt1 + j) & 1, p.ctl, ab))) break;
-          if (j == 0 && r > 0 && !(ok = mbar_wait_warp(bar_oe + 8, (r - 1) & 1, p.ctl, ab))) break;
+          if (j == 0 && n1 > 0 && !(ok = mbar_wait_warp(bar_oe + 8, (n1 - 1) & 1, p.ctl, ab))) break;
           tc_fence_after();
           issue_pv(1, vpos, j > 0, 0);
           if (!(ok = mbar_wait_warp(bar_p + 24, (cnt1 + j) & 1, p.ctl, ab))) break;
@@ -734,11 +1016,15 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
               if (!(ok = wait_slot(vpos + 2))) break;
             }
             if (j + 2 == nt) tc_commit_el(bar_qe + 8);  // tile 1's last S of the item
+            if (SPLIT && j + 2 == nt) tc_commit_el(bar_done);
           }
         }
+        if (!ok) break;
         cnt0 += nt0;
         cnt1 += nt;
         pos += 2 * nt;
+        n0 += !ONE || nt0 > 0;
+        ++n1;
       }
       // wait for every MMA issued above before TMEM may be released
       Abort no_abort{ab.flag + 1};
@@ -764,15 +1050,20 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     const int off = p.Skv - p.Sq;
 
     int cnt = 0;  // S tiles of this query tile processed in earlier items
+    int n0 = 0, n1 = 0;  // items so far that had a tile 0, a tile 1
+    int n_active = 0;    // SPLIT: items so far that had this tile in any CTA of the cluster
     bool ok = true;
     SeqCursor cur = VARLEN ? seq_cursor<kRows>(p) : SeqCursor{0, 0, 0};
-    for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur)) >= 0; ++r) {
-      const Item it = make_item_t<D, VARLEN>(p, cur, idx);
-      const int row = it.q0 + t * C::BM + row_in_tile;
+    for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur, wk, n_wk)) >= 0; ++r) {
+      const Item it = item_of(cur, idx);
+      const int row = (t == 0 ? it.q0 : it.q1) + row_in_tile;
       const int skv = VARLEN ? it.skv : p.Skv;
       const int offv = VARLEN ? it.skv - it.sq : off;
-      const int limit = p.causal ? min(skv, row + offv + 1) : skv;  // keys [0, limit) visible
+      const int query = VARLEN ? row : row >> p.pack_log2;
+      const int limit =
+          (p.causal ? min(skv, query + offv + 1) : skv) - (SPLIT ? it.kt0 * C::BN : 0);  // keys [0, limit) visible
       const int my_tiles = t == 0 ? it.n_tiles0 : it.n_tiles;
+      const int my_n = t == 0 ? n0 : n1;
       float m_run = -INFINITY, l_run = 0.f;
       for (int j = 0; ok && j < my_tiles; ++j)
         ok = softmax_step<D, C::BN, true>(s_tm, o_tm, my_bar_s, (cnt + j) & 1, my_bar_p, my_bar_o,
@@ -780,12 +1071,28 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
                                     l_run, p.ctl, ab);
       if (!ok) break;
       // epilogue: hand O_t back to the MMA warp, O / l -> bf16 rows, LSE
-      if (!(ok = softmax_epilogue<D, VARLEN>(o_tm, my_bar_o, r & 1, my_bar_oe, m_run,
-                                             l_run, row, it.q_z, p, ab, &tm_o, stg_q,
-                                             VARLEN ? it.qb : 0, VARLEN ? it.sq : 0, bar_mine, bar_peer,
-                                             t == 1 ? r & 1 : (r - 1) & 1, C::SHARED_STG && (t == 1 || r > 0))))
-        break;
+      if constexpr (SPLIT > 0) {
+        // (a tile of the item may still have no KV tiles in this CTA)
+        const bool active = t == 1 || it.q1 != it.q0;
+        const SplitRow sr{p.o, p.lse, p.Sq, p.q_rows, p.pack_log2, row, it.q_z, m_run, l_run, my_tiles > 0, active,
+                          r == 0, static_cast<uint32_t>(my_n & 1), static_cast<uint32_t>(r & 1),
+                          static_cast<uint32_t>(n_active & 1)};
+        const SplitBars sb{my_bar_o, my_bar_oe, bar_rdy, bar_xf, bar_xdone};
+        if (!(ok = split_epilogue<D, S>(sr, sb, o_tm, sbase,
+                                        sbase + C::STG_OFF + static_cast<uint32_t>(warp) * 4096u, warp, rank, p.ctl, ab)))
+          break;
+        n_active += active;
+      } else if (!ONE || my_tiles > 0) {
+        // shared staging: tile 0's release in this item, or tile 1's in the item before
+        if (!(ok = softmax_epilogue<D, VARLEN, !VARLEN>(
+                  o_tm, my_bar_o, my_n & 1, my_bar_oe, m_run, l_run, row, it.q_z, p, ab, &tm_o, stg_q,
+                  VARLEN ? it.qb : 0, VARLEN ? it.sq : 0, bar_mine, bar_peer, t == 1 ? n0 & 1 : (n1 - 1) & 1,
+                  C::SHARED_STG && (t == 1 ? !ONE || it.n_tiles0 > 0 : n1 > 0))))
+          break;
+      }
       cnt += my_tiles;
+      n0 += !ONE || it.n_tiles0 > 0;
+      n1 += !SPLIT || it.n_tiles > 0;
     }
     if (lane == 0) bulk_wait_group0();  // the O stores have completed before the CTA exits
   }
@@ -797,6 +1104,7 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);
   }
+  if constexpr (SPLIT > 0) cluster_sync_all();  // no peer writes to a CTA that has left
 }
 
 // ---------------------------------------------------------------- single-tile variant
@@ -1687,6 +1995,24 @@ bool make_map_tokens(CUtensorMap* map, const void* base, int D, int H, int total
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 4-D view [planes, Sq, 2^pack_log2, D] of a [B, H, S, D] bf16 tensor whose planes are
+// 2^pack_log2 heads each (innermost first: D, heads, rows, planes) with a box of box_rows
+// packed rows (row i: query i >> pack_log2 of head i mod 2^pack_log2), which lands in shared
+// memory like the dense 64 x box_rows box.
+bool make_map_packed(CUtensorMap* map, const void* base, int D, int Sq, int planes, int pack_log2, int box_rows) {
+  EncodeTiledFn enc = get_encode_fn();
+  if (!enc) return false;
+  const cuuint64_t row = static_cast<cuuint64_t>(D) * 2, head = row * static_cast<cuuint64_t>(Sq);
+  cuuint64_t dims[4] = {static_cast<cuuint64_t>(D), 1ull << pack_log2, static_cast<cuuint64_t>(Sq),
+                        static_cast<cuuint64_t>(planes)};
+  cuuint64_t strides[3] = {head, row, head << pack_log2};
+  cuuint32_t box[4] = {64, 1u << pack_log2, static_cast<cuuint32_t>(box_rows) >> pack_log2, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // A launch, as a programmatic dependent of the previous kernel in the stream
 // (cudaLaunchAttributeProgrammaticStreamSerialization) when `dependent`: the prefill
 // kernels wait for that kernel (griddepcontrol.wait) after their set-up and before any
@@ -1756,16 +2082,118 @@ cudaError_t launch_varlen_d(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaSt
   return launch_dependent(false, attn_fwd_kernel<D, true>, grid, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
 }
 
+// Query heads of one kv head packed into a plane of the two-tile design (as a power of two):
+// the largest that divides the group, up to the 32 rows of a warp.  Packed rows are ordered
+// by query, so a tile's rows span few queries: chunks of a few queries fill whole tiles (Sq
+// 515, G 4: 9 pairs per kv head instead of 12) and every pair of a causal item ends at the
+// same KV tile.
+int fwd_pack_log2(int G, int Sq) {
+  int lg = 0;
+  while (lg < 5 && (G >> lg) % 2 == 0 && Sq <= (0x3fffffff >> (lg + 1))) ++lg;
+  return lg;
+}
+
+// Clusters of S two-tile CTAs resident on the current device at once; 0 if none or unknown.
+// Cached per device and size.
+template <int D, int S>
+int fwd_max_clusters(int dev) {
+  using C = FwdCfg<D>;
+  static std::atomic<int> cache[64];  // value + 1 once known
+  static PerDeviceOnce configured;
+  if (dev < 0 || dev >= 64) return 0;
+  const int c = cache[dev].load(std::memory_order_relaxed);
+  if (c != 0) return c - 1;
+  int clusters = 0;
+  if (configured.run(dev, [] {
+        return cudaFuncSetAttribute(attn_fwd_kernel<D, false, 0, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    C::BYTES) == cudaSuccess;
+      })) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(S) * 64);
+    cfg.blockDim = dim3(C::THREADS);
+    cfg.dynamicSmemBytes = C::BYTES;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(S);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&clusters, attn_fwd_kernel<D, false, 0, S>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      clusters = 0;
+    }
+  }
+  cache[dev].store(clusters + 1, std::memory_order_relaxed);
+  return clusters;
+}
+
+template <int D>
+int fwd_max_clusters(int dev, int S) {
+  return S == 2 ? fwd_max_clusters<D, 2>(dev) : S == 4 ? fwd_max_clusters<D, 4>(dev) : fwd_max_clusters<D, 8>(dev);
+}
+
+// CTAs per cluster that share an item's KV tiles (1: no cluster): the lowest estimate of
+//   the busiest worker's items x (KV-tile steps of its share + boundary)
+// over 1, 2, 4 and 8.  In a launch with few items the SMs without one idle while the others
+// walk all keys in turn.  GB300, us on the device, S = 1 / 2 / 4 / 8 (D = 128 unless said):
+//   Sq 515 of Skv 3001, Hq 32, Hkv 8   37.8 / 27.5 / 40.6 / 80.8   (72 items: 76 clusters of 2 fit)
+//   Sq 128 of 4096, Hq 32, Hkv 8       47.2 / 31.7 / 22.8 / 37.2
+//   Sq 300 of 16384, Hq 8, Hkv 1        170 /   94 /   55 /   38
+//   S 4096 causal, Hq 8, Hkv 1         48.1 / 38.3 / 63.9 /  135   (two rounds of clusters)
+//   S 1024, H 8                        15.8 / 15.8 / 16.5 / 16.2
+//   S 1500, H 32 (192 items)           39.9 / 51.4 / 87.9 /    -
+// From these: a step of a pair of tiles takes kStep, an item's boundary kItem, with an
+// exchange kExchange more plus kPerDoubling for every doubling of the cluster.
+template <int D>
+int fwd_split(const FwdParams& p, int sms, int dev) {
+  constexpr double kStep = D == 128 ? 1330.0 : 1200.0;  // ns
+  constexpr double kItem = 3000.0, kExchange = 2500.0, kPerDoubling = 3000.0;
+  if (p.n_items >= 2 * sms) return 1;
+  const int planes = p.n_items / p.n_pairs;
+  const long long all = (p.Skv + 127) / 128;
+  int best = 1;
+  double best_t = 0.0;
+  for (int S = 1, doublings = 0; S <= 8 && all >= 2 * (S > 1 ? S : 0); S *= 2, ++doublings) {  // two tiles a CTA or more
+    const int fit = S == 1 ? sms : fwd_max_clusters<D>(dev, S);
+    if (fit < 1) continue;
+    const int workers = p.n_items < fit ? p.n_items : fit;
+    const int rounds = (p.n_items + workers - 1) / workers;
+    const double edge = kItem + (S > 1 ? kExchange + kPerDoubling * doublings : 0.0);
+    auto cost = [&](long long tiles) { return static_cast<double>((tiles + S - 1) / S) * kStep + edge; };
+    double t = rounds * cost(all);
+    if (p.causal) {  // items of different lengths, dealt evenly: the average, the longest, all of the shortest
+      double total = 0.0, shortest = 0.0;
+      for (int i = 0; i < p.n_pairs; ++i) {
+        const long long kv = ((256ll * (i + 1)) >> p.pack_log2) + (p.Skv - p.Sq);
+        const double c = cost(((kv < p.Skv ? kv : p.Skv) + 127) / 128);
+        if (i == 0) shortest = c;
+        total += c;
+      }
+      t = total * planes / workers;
+      if (t < cost(all)) t = cost(all);
+      if (t < rounds * shortest) t = rounds * shortest;
+    }
+    if (S == 1 || t < best_t * (best == 1 ? 0.95 : 1.0)) {
+      best = S;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
 // Launch one design: C is its configuration, rows_per_item the query rows of one work
-// item (C::NQT * C::BM).
-template <int D, class C, class Kernel>
+// item (C::NQT * C::BM).  PACKED: the two-tile design over planes of packed heads.
+template <int D, class C, bool PACKED = false, class Kernel>
 cudaError_t launch_design(Kernel kernel, int rows_per_item, const FwdArgs& a, const KernelCtl& ctl,
                           cudaStream_t stream, PerDeviceOnce& configured) {
+  const int lg = PACKED ? fwd_pack_log2(a.Hq / a.Hkv, a.Sq) : 0;
+  const int planes = (a.B * a.Hq) >> lg;
   CUtensorMap mq, mk, mv, mo;
-  if (!make_map(&mq, a.q, D, a.Sq, a.B * a.Hq, C::BM) ||
-      !make_map(&mk, a.k, D, a.Skv, a.B * a.Hkv, C::BN) ||
-      !make_map(&mv, a.v, D, a.Skv, a.B * a.Hkv, C::BN) ||
-      !make_map(&mo, a.o, D, a.Sq, a.B * a.Hq, 32))  // epilogue: one 32-row block per warp
+  if (PACKED ? !make_map_packed(&mq, a.q, D, a.Sq, planes, lg, C::BM) ||
+                   !make_map_packed(&mo, a.o, D, a.Sq, planes, lg, 32)
+             : !make_map(&mq, a.q, D, a.Sq, planes, C::BM) || !make_map(&mo, a.o, D, a.Sq, planes, 32))
+    return cudaErrorInvalidValue;  // (O leaves in one 32-row block per warp)
+  if (!make_map(&mk, a.k, D, a.Skv, a.B * a.Hkv, C::BN) || !make_map(&mv, a.v, D, a.Skv, a.B * a.Hkv, C::BN))
     return cudaErrorInvalidValue;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1774,27 +2202,55 @@ cudaError_t launch_design(Kernel kernel, int rows_per_item, const FwdArgs& a, co
       }))
     return cudaErrorInvalidValue;
   FwdParams p;
+  memset(&p, 0, sizeof(p));
   p.o = static_cast<__nv_bfloat16*>(a.o);
   p.lse = a.lse;
   p.Hq = a.Hq;
   p.Hkv = a.Hkv;
   p.Sq = a.Sq;
   p.Skv = a.Skv;
-  p.n_pairs = (a.Sq + rows_per_item - 1) / rows_per_item;
+  p.pack_log2 = lg;
+  p.planes_per_kv = (a.Hq / a.Hkv) >> lg;
+  p.q_rows = a.Sq << lg;
+  p.n_pairs = (p.q_rows + rows_per_item - 1) / rows_per_item;
   p.causal = a.causal;
   p.c = a.scale * kLog2e;
   p.ctl = ctl;
-  const long long items = static_cast<long long>(p.n_pairs) * a.B * a.Hq;
+  const long long items = static_cast<long long>(p.n_pairs) * planes;
   if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   p.n_items = static_cast<int>(items);
-  // (the block layout is set below, once the grid is known)
   // persistent: one CTA per SM (shared memory / TMEM admit one), each walking its items
   int sms = 0;
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int grid = static_cast<int>(items < sms ? items : sms);
-  p.plane_block = model::causal_block_layout(a.B * a.Hq, a.Hq / a.Hkv, a.Skv, D, p.n_pairs, grid, &p.last_h0);
-  return launch_dependent(!a.causal, kernel, grid, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
+  int S = 1;
+  if constexpr (PACKED) {
+    if (a.slots == 0) S = fwd_split<D>(p, sms, dev);
+  }
+  const int fit = S > 1 ? fwd_max_clusters<D>(dev, S) : sms;
+  const int workers = static_cast<int>(items < fit ? items : fit);
+  p.plane_block =
+      model::causal_block_layout(planes, (a.Hq / a.Hkv) >> lg, a.Skv, D, p.n_pairs, workers, &p.last_h0);
+  if constexpr (PACKED) {
+    if (S > 1) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(static_cast<unsigned>(workers * S));
+      cfg.blockDim = dim3(C::THREADS);
+      cfg.dynamicSmemBytes = C::BYTES;
+      cfg.stream = stream;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = static_cast<unsigned>(S);
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      auto split_kernel = S == 2   ? attn_fwd_kernel<D, false, 0, 2>
+                          : S == 4 ? attn_fwd_kernel<D, false, 0, 4>
+                                   : attn_fwd_kernel<D, false, 0, 8>;
+      return cudaLaunchKernelEx(&cfg, split_kernel, mq, mk, mv, mo, p);
+    }
+  }
+  return launch_dependent(!a.causal, kernel, workers, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
 }
 
 // Ring depths compiled for the block-size ablation of the two-tile design (the model's
@@ -1805,12 +2261,12 @@ cudaError_t launch_two_tile_slots(const FwdArgs& a, const KernelCtl& ctl, cudaSt
   constexpr int kRows = FwdCfg<D>::NQT * FwdCfg<D>::BM;
   if constexpr (D == 128) {
     static PerDeviceOnce once2;
-    if (a.slots == 2) return launch_design<D, FwdCfg<D, 2>>(attn_fwd_kernel<D, false, 2>, kRows, a, ctl, stream, once2);
+    if (a.slots == 2) return launch_design<D, FwdCfg<D, 2>, true>(attn_fwd_kernel<D, false, 2>, kRows, a, ctl, stream, once2);
   } else {
     static PerDeviceOnce once3, once6, once9;
-    if (a.slots == 3) return launch_design<D, FwdCfg<D, 3>>(attn_fwd_kernel<D, false, 3>, kRows, a, ctl, stream, once3);
-    if (a.slots == 6) return launch_design<D, FwdCfg<D, 6>>(attn_fwd_kernel<D, false, 6>, kRows, a, ctl, stream, once6);
-    if (a.slots == 9) return launch_design<D, FwdCfg<D, 9>>(attn_fwd_kernel<D, false, 9>, kRows, a, ctl, stream, once9);
+    if (a.slots == 3) return launch_design<D, FwdCfg<D, 3>, true>(attn_fwd_kernel<D, false, 3>, kRows, a, ctl, stream, once3);
+    if (a.slots == 6) return launch_design<D, FwdCfg<D, 6>, true>(attn_fwd_kernel<D, false, 6>, kRows, a, ctl, stream, once6);
+    if (a.slots == 9) return launch_design<D, FwdCfg<D, 9>, true>(attn_fwd_kernel<D, false, 9>, kRows, a, ctl, stream, once9);
   }
   *handled = false;
   return cudaSuccess;
@@ -1839,7 +2295,12 @@ cudaError_t launch_fwd_d(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t st
       return launch_design<D, Fwd4Cfg<D>>(attn_fwd4_kernel<D>, Fwd4Cfg<D>::NQT * Fwd4Cfg<D>::BM, a, ctl,
                                           stream, configured4);
   }
-  return launch_design<D, FwdCfg<D>>(attn_fwd_kernel<D>, FwdCfg<D>::NQT * FwdCfg<D>::BM, a, ctl, stream,
+  static PerDeviceOnce configured_one;
+  constexpr int kRows = FwdCfg<D>::NQT * FwdCfg<D>::BM;
+  const long long last = (static_cast<long long>(a.Sq) << fwd_pack_log2(a.Hq / a.Hkv, a.Sq)) % kRows;
+  if (last > 0 && last <= FwdCfg<D>::BM)  // a plane's last item has one query tile
+    return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D>, kRows, a, ctl, stream, configured_one);
+  return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D, false, 0, 0, false>, FwdCfg<D>::NQT * FwdCfg<D>::BM, a, ctl, stream,
                                      configured2);
 }
 

@@ -1,0 +1,92 @@
+"""GPU parity of the prefill paths that few work items take: heads packed into planes of
+query rows, items of one query tile, and clusters of CTAs that share an item's KV tiles."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from tests.gpu_util import assert_parity, o_to_f64, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def loom():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2609_29219_gb300 as m
+    return m
+
+
+# B, Hq, Hkv, Sq, Skv, D, causal: clusters of 2 with a one-tile item last in its plane; of 4
+# with 1000 + 1 rows of G = 2; of 8 with a handful of rows; several items per cluster; a
+# share that ends before tile 0's diagonal; groups that are no power of two; no causal mask
+SHAPES = [
+    (1, 32, 8, 515, 3001, 128, True), (2, 6, 3, 700, 2000, 128, True), (1, 8, 1, 3, 4100, 128, True),
+    (1, 8, 1, 300, 2049, 64, True), (1, 8, 8, 2048, 2048, 128, True), (1, 4, 4, 1500, 1500, 64, True),
+    (1, 6, 1, 130, 2300, 128, False), (2, 4, 4, 129, 5000, 64, False), (1, 32, 1, 65, 1025, 128, True),
+    (1, 12, 1, 129, 4096, 64, True), (3, 16, 4, 257, 2600, 128, False),
+]
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,causal", SHAPES)
+def test_few_items(loom, B, Hq, Hkv, Sq, Skv, D, causal):
+    import torch
+    q = synth.bf16_normal(1, synth.STREAM_Q, (B, Hq, Sq, D))
+    k = synth.bf16_normal(1, synth.STREAM_K, (B, Hkv, Skv, D))
+    v = synth.bf16_normal(1, synth.STREAM_V, (B, Hkv, Skv, D))
+    o = torch.full((B, Hq, Sq, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((B, Hq, Sq), float("nan"), device="cuda")
+    # a second call on the same buffers gives the same bits: nothing depends on timing
+    loom.loom_attn_fwd(to_dev(q), to_dev(k), to_dev(v), o, lse, causal=causal)
+    first = o.clone(), lse.clone()
+    loom.loom_attn_fwd(to_dev(q), to_dev(k), to_dev(v), o, lse, causal=causal)
+    loom.loom_attn_check_error()
+    assert torch.equal(o.view(torch.int16), first[0].view(torch.int16)) and torch.equal(lse, first[1])
+    o_ref, lse_ref = oracle.attention(q, k, v, causal=causal)
+    assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy(), lse_ref, f"{(B, Hq, Hkv, Sq, Skv, D, causal)}")
+
+
+def test_extreme_scores_across_shares(loom):
+    """Rows whose largest scores lie in one CTA's share: the other shares' weights underflow
+    to zero (their partials must not bring in NaN or infinity)."""
+    B, Hq, Hkv, Sq, Skv, D = 1, 4, 1, 64, 4096, 64
+    q = synth.bf16_normal(2, synth.STREAM_Q, (B, Hq, Sq, D))
+    k = synth.bf16_normal(2, synth.STREAM_K, (B, Hkv, Skv, D))
+    v = synth.bf16_normal(2, synth.STREAM_V, (B, Hkv, Skv, D))
+    kf = (k.astype(np.uint32) << 16).view(np.float32).copy()
+    kf[:, :, :700] *= 60.0
+    k = synth.f32_to_bf16(kf)
+    o, lse = loom.loom_attn_fwd(to_dev(q), to_dev(k), to_dev(v), return_lse=True)
+    loom.loom_attn_check_error()
+    o_ref, lse_ref = oracle.attention(q, k, v)
+    assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy(), lse_ref, "scores of one share dominate")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_timeout_in_a_cluster_is_reported(loom, D):
+    """A K/V tile that never arrives in any CTA of a cluster: every wait runs out, the call
+    reports it, and the next call is right."""
+    B, Hq, Hkv, Sq, Skv = 1, 8, 2, 200, 4000
+    q = synth.bf16_normal(3, synth.STREAM_Q, (B, Hq, Sq, D))
+    k = synth.bf16_normal(3, synth.STREAM_K, (B, Hkv, Skv, D))
+    v = synth.bf16_normal(3, synth.STREAM_V, (B, Hkv, Skv, D))
+    qd, kd, vd = to_dev(q), to_dev(k), to_dev(v)
+    loom.loom_attn_check_error()
+    loom.loom_debug_set_timeout_ns(50_000_000)
+    try:
+        loom.loom_debug_inject(2)
+        loom.loom_attn_fwd(qd, kd, vd)
+        with pytest.raises(loom.LoomError) as e:
+            loom.loom_attn_check_error()
+        assert e.value.status == 6
+    finally:
+        loom.loom_debug_inject(0)
+        loom.loom_debug_set_timeout_ns(0)
+    o, lse = loom.loom_attn_fwd(qd, kd, vd, return_lse=True)
+    loom.loom_attn_check_error()
+    o_ref, lse_ref = oracle.attention(q, k, v)
+    assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy(), lse_ref, f"after timeout D={D}")
