@@ -101,7 +101,8 @@ int loom_attn_decode_num_splits(int B, int Hq, int Hkv, int Skv, int D);
  * Device workspace (bytes) that loom_attn_decode needs: the per-split partial outputs
  * O_i [B, Hq, splits, D] fp32 and log-sum-exps lse_i [B, Hq, splits] fp32 (each from a
  * 256-byte boundary), then 256 bytes holding the persistent split kernel's item counter.
- * num_splits = 0 means the model's choice.  Returns 0 on invalid sizes.
+ * num_splits = 0 means the model's choice, for B > 1 with room for a larger count where
+ * unequal lengths want one (see num_splits below).  Returns 0 on invalid sizes.
  */
 size_t loom_attn_decode_workspace_bytes(int B, int Hq, int Hkv, int Skv, int D, int num_splits);
 
@@ -118,7 +119,10 @@ size_t loom_attn_decode_workspace_bytes(int B, int Hq, int Hkv, int Skv, int D, 
  *              its contents on entry do not matter and are overwritten (the item
  *              counter in its last 256 bytes is left armed for the next call; a
  *              workspace serves one call at a time).
- *   num_splits 0 = analytic model, otherwise 1..1024 splits of each sequence.
+ *   num_splits 0 = analytic model, otherwise 1..1024 splits of each sequence.  With 0,
+ *              lengths that differ may take more splits than the model's count (of
+ *              loom_attn_decode_num_splits), decided on the device, if the workspace has
+ *              room for them; a workspace of that count is enough.
  * Split i of sequence b covers keys [i*C, min((i+1)*C, len_b)), C = ceil(len_b/splits)
  * rounded up to a multiple of 64; empty splits contribute nothing.  A sequence of
  * length 0 yields O = 0 and LSE = -inf.
@@ -186,7 +190,8 @@ loom_status loom_attn_decode_paged(const void* q, const void* k_cache, const voi
  * Arguments, layouts and results are those of loom_attn_decode.  The per-split partials
  * live in a scratch array built into the library (LOOM_DECODE_NOALLOC_SCRATCH_BYTES,
  * 8 MiB), held by every GPU that loads the library until the process exits.  A problem
- * whose partials need more (loom_attn_decode_workspace_bytes(...) larger than that)
+ * whose partials need more (loom_attn_decode_workspace_bytes(...) larger than that; with
+ * num_splits = 0, of the model's count loom_attn_decode_num_splits)
  * returns LOOM_ERR_WORKSPACE without launching anything.  The first call on a device
  * looks up the array's device address (cudaGetSymbolAddress, current device); make that
  * first call before any stream capture.  All calls share the array, which keeps the last

@@ -897,10 +897,45 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
 // the slot which item and which stage of it the slot holds; the MMA warp and the softmax
 // warp walk the ring and learn the item boundaries from those records, so neither needs
 // the counter.  A final record with b = -1 ends both.
+//
+// Splits of a ragged batch.  The model's split count is for sequences of one length; where
+// the lengths differ (which only the device knows) few items per CTA are as uneven as the
+// lengths: B16 of 4096 to 8192 keys at the model's 2 splits is 256 items on 304 CTAs, the
+// longest twice the shortest.  So the launch carries two counts, that one (`equal`) and a
+// larger one that the partials' space is laid out for (`splits`), and the kernels take the
+// larger one unless the mean length is within 4 % of the longest.  GB300, us, equal / larger
+// count, on unequal lengths and on equal ones (where more items only cost):
+//   B16 Hkv8 4096-8192         2 / 12: 75.0 / 68.1, paged by 16 keys 79.0 / 71.0
+//   B16 Hkv8 8192              2 / 12: 83.1 / 83.9 (2 splits either way: what choosing costs)
+// and not taken (see decode_ragged_splits):
+//   B64 Hkv8 512-2048          1 / 3: 71.1 / 68.3, equal lengths 91.9 / 92.7
+//   B4 Hkv8 4096-8192         8 / 16: 24.2 / 23.1, equal lengths 28.6 / 29.2
+// The split kernel's CTA 0 leaves its count behind the item counter for the merge kernel.
+// Splits of fewer than 65536 / D keys only cost (B48, 100 to 1000 keys: 2 -> 3 splits 31.2 ->
+// 32.4 us).
+
+// By the loader warp, from the B lengths in shared memory.
+__device__ __forceinline__ int ragged_splits(const int* lens, int B, int Skv, int D, int equal, int splits, int lane) {
+  float total = 0.f;
+  int longest = 0;
+  for (int b = lane; b < B; b += 32) {
+    const int n = max(0, min(lens[b], Skv));
+    total += static_cast<float>(n);
+    longest = max(longest, n);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    total += __shfl_xor_sync(0xffffffffu, total, off);
+    longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, off));
+  }
+  if (total >= 0.96f * static_cast<float>(longest) * static_cast<float>(B)) return equal;
+  return max(equal, min(splits, longest / (65536 / D)));
+}
+
 template <int D>
 struct DecodeTcPersistCfg {
   using C = DecodeTcCfg<D>;
-  static constexpr int kMaxSortedB = 256;                 // sequences sorted by length
+  static constexpr int kMaxSortedB = kMaxRaggedB;         // sequences sorted by length
   static constexpr uint32_t Q_BOX_BYTES = C::MAX_G * 128;  // up to 32 heads x 64 dims
   static constexpr uint32_t Q_OFF = C::NSTAGE * C::STAGE_BYTES;
   static constexpr uint32_t META_OFF = Q_OFF + C::NBOX * Q_BOX_BYTES;  // [NSTAGE] x 8 int32
@@ -923,7 +958,7 @@ struct DecodeTcPersistCfg {
 template <int D>
 __device__ __forceinline__ void decode_tc_persist_rows(const uint8_t* smem, float* __restrict__ o_part,
                                                        float* __restrict__ lse_part, uint32_t tmem, int G, int Hq,
-                                                       int splits, float c, uint32_t bar_full, uint32_t bar_qf,
+                                                       float c, uint32_t bar_full, uint32_t bar_qf,
                                                        uint32_t bar_qe, uint32_t bar_q, uint32_t bar_s, uint32_t bar_p,
                                                        uint32_t bar_o, const KernelCtl& ctl, const Abort& ab) {
   using C = DecodeTcCfg<D>;
@@ -938,7 +973,7 @@ __device__ __forceinline__ void decode_tc_persist_rows(const uint8_t* smem, floa
     const volatile int* rec = reinterpret_cast<const volatile int*>(smem + L::META_OFF + slot * 32);
     const int b = rec[0];
     if (b < 0) return;  // no more items
-    const int hk = rec[1], split = rec[2], j = rec[3], n_st = rec[4], ntok = rec[6];
+    const int hk = rec[1], split = rec[2], j = rec[3], n_st = rec[4], ntok = rec[6], splits = rec[7];
     if (j == 0) {
       if (!mbar_wait_warp(bar_qf, nq & 1, ctl, ab)) return;
 #pragma unroll
@@ -1044,7 +1079,7 @@ template <int D, bool PAGED>
 __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
     decode_tc_persist_kernel(const int32_t* __restrict__ seqlens, float* __restrict__ o_part,
                              float* __restrict__ lse_part, unsigned long long* __restrict__ sched, int B, int Hq,
-                             int Hkv, int Skv, int splits, float c, KernelCtl ctl, const __grid_constant__ CUtensorMap tm_q,
+                             int Hkv, int Skv, int splits, int equal, float c, KernelCtl ctl, const __grid_constant__ CUtensorMap tm_q,
                              const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                              PagedView pv) {
   using C = DecodeTcCfg<D>;
@@ -1057,8 +1092,6 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
   uint8_t* smem = smem_raw + (sbase - raw_base);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = Hq / Hkv;
-  const long long per_seq = static_cast<long long>(Hkv) * splits;
-  const long long n_items = B * per_seq;
 
   const uint32_t bar_full = sbase + L::BAR_OFF;
   const uint32_t bar_empty = bar_full + 8 * C::NSTAGE;
@@ -1100,6 +1133,7 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
   // the sequences in order of decreasing length (ties by index): items are taken in it
   int* order = reinterpret_cast<int*>(smem + L::ORDER_OFF);
   const bool sorted = seqlens != nullptr && B <= L::kMaxSortedB;
+  int count = splits;  // splits of every sequence
   if (sorted) {
     int* lens = reinterpret_cast<int*>(smem + L::LENS_OFF);
     for (int bb = threadIdx.x; bb < B; bb += blockDim.x) lens[bb] = seqlens[bb];
@@ -1112,6 +1146,11 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
         r += (lx > lb) || (lx == lb && x < bb);
       }
       order[r] = bb;
+    }
+    // (by the loader warp, while warp 0 sorts; equal > 0 implies sorted)
+    if (warp == 1 && equal > 0) {
+      count = ragged_splits(lens, B, Skv, D, equal, splits, lane);
+      if (blockIdx.x == 0 && lane == 0) sched[1] = static_cast<unsigned long long>(count);
     }
     __syncthreads();
   }
@@ -1131,6 +1170,8 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
     // workspace never armed (its first call) deals them statically, item blockIdx.x +
     // k * gridDim.x (every CTA reads the same unarmed tag: all take the same branch).
     unsigned long long ticket = lane == 0 ? atomicAdd(sched, 1ull) : 0ull;
+    const long long per_seq = static_cast<long long>(Hkv) * count;
+    const long long n_items = B * per_seq;
     int dynamic = -1;  // read from the first ticket once the first item is under way
     long long item = blockIdx.x;
     int st = 0, nq = 0, skipped = -1;
@@ -1142,19 +1183,19 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
       const int split = rem / Hkv, hk = rem - split * Hkv;
       int len = seqlens ? seqlens[b] : Skv;
       len = max(0, min(len, Skv));
-      int chunk = (len + splits - 1) / splits;
+      int chunk = (len + count - 1) / count;
       chunk = (chunk + kDecodeChunkAlign - 1) / kDecodeChunkAlign * kDecodeChunkAlign;
       const int t_begin = min(split * chunk, len);
       const int t_end = min(t_begin + chunk, len);
       if (t_begin >= t_end) {
         // empty split: contributes nothing to the merge
-        const size_t row0 = (static_cast<size_t>(b) * Hq + static_cast<size_t>(hk) * G) * splits + split;
+        const size_t row0 = (static_cast<size_t>(b) * Hq + static_cast<size_t>(hk) * G) * count + split;
         for (int i = lane; i < G * (D / 4); i += 32) {
           const int r = i / (D / 4);
-          reinterpret_cast<float4*>(o_part + (row0 + static_cast<size_t>(r) * splits) * D)[i % (D / 4)] =
+          reinterpret_cast<float4*>(o_part + (row0 + static_cast<size_t>(r) * count) * D)[i % (D / 4)] =
               make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        for (int r = lane; r < G; r += 32) lse_part[row0 + static_cast<size_t>(r) * splits] = -INFINITY;
+        for (int r = lane; r < G; r += 32) lse_part[row0 + static_cast<size_t>(r) * count] = -INFINITY;
       } else {
         // the item's q rows, once the softmax warp has moved the previous ones to TMEM
         if (!(ok = mbar_wait_warp(bar_qe, (nq & 1) ^ 1, ctl, ab))) break;
@@ -1186,6 +1227,7 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
             rec[4] = n_st;
             rec[5] = tok0;
             rec[6] = ntok;
+            rec[7] = count;
           }
           if constexpr (PAGED) {
             // pieces of min(page, 64) keys: a stage starts on a multiple of 64, so a piece
@@ -1295,7 +1337,7 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
     mbar_wait_warp(bar_drain, 0, ctl, no_abort);
   } else {
     // ------------------------------------------------------------ softmax (warp 0)
-    decode_tc_persist_rows<D>(smem, o_part, lse_part, tmem, G, Hq, splits, c, bar_full, bar_qf, bar_qe, bar_q, bar_s,
+    decode_tc_persist_rows<D>(smem, o_part, lse_part, tmem, G, Hq, c, bar_full, bar_qf, bar_qe, bar_q, bar_s,
                               bar_p, bar_o, ctl, ab);
   }
 
@@ -1620,12 +1662,16 @@ __global__ void __launch_bounds__(DecodeCfg<D>::THREADS, DecodeCfg<D>::CTAS_PER_
 // One CTA (D threads) per (batch, query head).  The split log-sum-exps are read in
 // parallel (one per thread), reduced, turned into weights in shared memory, and the
 // partial rows are streamed with 8 independent loads in flight per thread.
-template <int D>
+// RAGGED: the split kernel has left its split count (`equal` or more, `splits` at most, which
+// is kMergeRegSplits at most) behind the item counter.  A kernel of its own: with the count
+// a run-time value everywhere, the plain merge lost 1 us on B16, 2 us on B64.
+constexpr int kMergeRegSplits = 64;
+template <int D, bool RAGGED>
 __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict__ o_part,
                                                          const float* __restrict__ lse_part,
                                                          __nv_bfloat16* __restrict__ o,
                                                          float* __restrict__ lse, int splits,
-                                                         unsigned long long* __restrict__ sched) {
+                                                         unsigned long long* __restrict__ sched, int equal) {
   constexpr int NW = D / 32;
   __shared__ float w_s[kMaxDecodeSplits];
   __shared__ float red[NW];
@@ -1638,13 +1684,15 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
   if (sched != nullptr && blockIdx.x == 0 && threadIdx.x == 0)
     *sched = static_cast<unsigned long long>(kDecodeSchedTag) << 32;
   const int bh = blockIdx.x, d = threadIdx.x, lane = d & 31, wid = d >> 5;
+  // RAGGED: the partials of `equal` splits are requested without waiting for the count
+  const int most = splits;
+  if constexpr (RAGGED) splits = equal;
   const float* lp = lse_part + static_cast<size_t>(bh) * splits;
   const float* op = o_part + static_cast<size_t>(bh) * splits * D + d;
   // Up to kMergeRegSplits splits, every partial of this thread's dimension is requested
   // before the weights are known, so the merge waits for one round trip to memory
   // instead of one per reduction step and per batch of partials.
-  constexpr int kMergeRegSplits = 64;
-  const bool in_regs = splits <= kMergeRegSplits;
+  const bool in_regs = RAGGED || splits <= kMergeRegSplits;
   float pre[kMergeRegSplits];
   if (in_regs) {
 #pragma unroll
@@ -1652,7 +1700,22 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
   }
 
   float m = -INFINITY;
-  for (int i = d; i < splits; i += D) m = fmaxf(m, lp[i]);
+  if constexpr (RAGGED) {
+    static_assert(kMergeRegSplits <= D, "a split's LSE per thread");
+    if (d < splits) m = lp[d];
+    const int count = min(most, static_cast<int>(__ldcg(sched + 1)));
+    if (count != splits) {
+      splits = count;
+      lp = lse_part + static_cast<size_t>(bh) * splits;
+      op = o_part + static_cast<size_t>(bh) * splits * D + d;
+      m = d < splits ? lp[d] : -INFINITY;
+#pragma unroll
+      for (int i = 0; i < kMergeRegSplits; ++i) pre[i] = i < splits ? op[static_cast<size_t>(i) * D] : 0.f;
+    }
+  } else {
+    for (int i = d; i < splits; i += D) m = fmaxf(m, lp[i]);
+  }
+  const float lse_mine = m;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
   if (lane == 0) red[wid] = m;
@@ -1664,7 +1727,7 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
 
   float ws = 0.f;
   for (int i = d; i < splits; i += D) {
-    const float w = (M == -INFINITY) ? 0.f : ex2((lp[i] - M) * kLog2e);  // 0 for empty splits
+    const float w = (M == -INFINITY) ? 0.f : ex2(((RAGGED ? lse_mine : lp[i]) - M) * kLog2e);  // 0 for empty splits
     w_s[i] = w;
     ws += w;
   }
@@ -1976,7 +2039,7 @@ cudaError_t launch_tc_persist(const DecodeArgs& a, const PagedKV* pk, const Kern
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, decode_tc_persist_kernel<D, PAGED>, a.seqlens, a.o_part, a.lse_part, a.sched, a.B,
-                            a.Hq, a.Hkv, a.Skv, a.splits, a.scale * kLog2e, ctl, tq, tk, tv, view);
+                            a.Hq, a.Hkv, a.Skv, a.splits, a.equal_splits, a.scale * kLog2e, ctl, tq, tk, tv, view);
 }
 
 template <int D, int GT, bool PAGED, bool CLUSTER>
@@ -2036,9 +2099,9 @@ cudaError_t launch_merge(const DecodeArgs& a, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_merge_kernel<D>, static_cast<const float*>(a.o_part),
+  return cudaLaunchKernelEx(&cfg, a.equal_splits > 0 ? decode_merge_kernel<D, true> : decode_merge_kernel<D, false>, static_cast<const float*>(a.o_part),
                             static_cast<const float*>(a.lse_part),
-                            static_cast<__nv_bfloat16*>(a.o), a.lse, a.splits, a.sched);
+                            static_cast<__nv_bfloat16*>(a.o), a.lse, a.splits, a.sched, a.equal_splits);
 }
 
 // The Flash Decode form of a launch: kDecodeSplitMerge, kDecodePersistent (both with the
@@ -2056,8 +2119,9 @@ int decode_form(const DecodeArgs& a, int* cs_out) {
                                                 cudaSuccess)
     return kDecodeSplitMerge;
   const int slots = persistent_slots<D, GT, PAGED>();
+  const int splits = a.equal_splits > 0 ? a.equal_splits : a.splits;
   const model::DecodeClusterChoice ch = model::choose_decode_cluster(
-      a.splits, a.B, a.Hq, a.Hkv, a.Skv, D, [](int cs) { return max_clusters<D, GT, PAGED>(cs); }, a.cluster);
+      splits, a.B, a.Hq, a.Hkv, a.Skv, D, [](int cs) { return max_clusters<D, GT, PAGED>(cs); }, a.cluster);
   if (a.form == kDecodeSplitMerge) return kDecodeSplitMerge;
   if (a.form == kDecodePersistent && slots > 0) return kDecodePersistent;
   if (a.form == kDecodeCluster && ch.cs > 0) {
@@ -2068,10 +2132,10 @@ int decode_form(const DecodeArgs& a, int* cs_out) {
   // such, and the CUDA-core persistent split kernel (the same schedule with a slower
   // stage, measured slower or equal on every shape) is not a candidate.
   const bool tc = decode_tc_eligible(a) && !(PAGED && a.tc == 2);
-  const double t_split = tc ? model::decode_tc_time_us(a.splits, a.B, a.Hq, a.Hkv, a.Skv, D, sms)
-                            : model::decode_time_us(a.splits, a.B, a.Hq, a.Hkv, a.Skv, D, sms);
+  const double t_split = tc ? model::decode_tc_time_us(splits, a.B, a.Hq, a.Hkv, a.Skv, D, sms)
+                            : model::decode_time_us(splits, a.B, a.Hq, a.Hkv, a.Skv, D, sms);
   const double t_persist =
-      (slots > 0 && !tc) ? model::decode_persistent_time_us(a.splits, a.B, a.Hq, a.Hkv, a.Skv, D, slots) : 1e300;
+      (slots > 0 && !tc) ? model::decode_persistent_time_us(splits, a.B, a.Hq, a.Hkv, a.Skv, D, slots) : 1e300;
   int form = kDecodeSplitMerge;
   double best = t_split;
   if (t_persist < best * (1.0 - 1e-9)) {
@@ -2113,10 +2177,17 @@ cudaError_t launch_ablation(const DecodeArgs& a, const KernelCtl& ctl, cudaStrea
 }
 
 template <int D, int GT, bool PAGED>
-cudaError_t launch_form(const DecodeArgs& a, const PagedKV* pk, const KernelCtl& ctl, cudaStream_t stream) {
+cudaError_t launch_form(const DecodeArgs& args, const PagedKV* pk, const KernelCtl& ctl, cudaStream_t stream) {
+  DecodeArgs a = args;
   if (D == 128 && GT == 4 && !PAGED && a.stage_plan > 0) return launch_ablation(a, ctl, stream);
   int cs = 0;
   const int form = decode_form<D, GT, PAGED>(a, &cs);
+  const bool tc_persist =
+      form == kDecodeSplitMerge && decode_tc_eligible(a) && a.tc != 2;  // counts splits by the lengths
+  if (!tc_persist && a.equal_splits > 0) {
+    a.splits = a.equal_splits;
+    a.equal_splits = 0;
+  }
   if (form == kDecodeCluster) return launch_cluster<D, GT, PAGED>(a, cs, pk, ctl, stream);
   cudaError_t e;
   if (form == kDecodePersistent)

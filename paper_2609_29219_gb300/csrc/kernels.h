@@ -53,7 +53,26 @@ struct DecodeArgs {
   int tc;          // split + merge form's split kernel on a contiguous cache: 0 CUDA cores; tensor
                    // cores, 1 persistent CTAs taking items from the workspace counter, 2 one CTA per split
   unsigned long long* sched;  // the workspace's item counter (tag kDecodeSchedTag in the high word)
+  int equal_splits;  // > 0: `splits` is decode_ragged_splits' count and this one the model's; the
+                     // kernels choose by the lengths (0: `splits` it is)
 };
+
+// Split count that the workspace of a call with the model's count `equal` is laid out for: up
+// to five items for each of the 304 CTAs, so that unequal lengths even out, of 65536 / D keys
+// or more.  Only where a sequence has few items and they fill one round: with more of either
+// the dealing evens the lengths out already, and unequal lengths gain no more than the second
+// count costs equal ones (see ragged_splits in attn_decode.cu for the measurements).
+constexpr int kMaxRaggedB = 256;  // sequences
+inline int decode_ragged_splits(int B, int Hq, int Hkv, int Skv, int D, int equal) {
+  if (B < 2 || B > kMaxRaggedB || Hq / Hkv > 32) return equal;
+  const long long units = static_cast<long long>(B) * Hkv;
+  if (units * equal > 304 || equal > 4) return equal;
+  long long r = (1536 + units - 1) / units;
+  const long long most = static_cast<long long>(Skv) * D / 65536;
+  if (r > most) r = most;
+  if (r > 64) r = 64;  // the merge holds them in registers
+  return r > equal ? static_cast<int>(r) : equal;
+}
 
 // High word of an armed item counter: a signalling-NaN pattern that no float the decode
 // path writes to the workspace carries, so that a workspace never used before is told

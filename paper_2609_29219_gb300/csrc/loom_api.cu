@@ -158,7 +158,10 @@ int loom_attn_decode_num_splits(int B, int Hq, int Hkv, int Skv, int D) {
 }
 
 size_t loom_attn_decode_workspace_bytes(int B, int Hq, int Hkv, int Skv, int D, int num_splits) {
-  if (num_splits == 0) num_splits = loom_attn_decode_num_splits(B, Hq, Hkv, Skv, D);
+  if (num_splits == 0) {
+    num_splits = loom_attn_decode_num_splits(B, Hq, Hkv, Skv, D);
+    if (num_splits > 0) num_splits = decode_ragged_splits(B, Hq, Hkv, Skv, D, num_splits);
+  }
   if (num_splits <= 0 || num_splits > kMaxDecodeSplits) return 0;
   if (B <= 0 || Hq <= 0 || (D != 64 && D != 128)) return 0;
   return decode_workspace_bytes(B, Hq, D, num_splits);
@@ -192,6 +195,20 @@ int decode_check_args(const void* q, const void* k_cache, const void* v_cache, c
   *splits = num_splits;
   return LOOM_OK;
 }
+
+namespace {
+// With the model's count and lengths on the device, lays the partials out for the larger
+// count of a ragged batch where the workspace holds it: *splits becomes that count and the
+// model's is returned (0: nothing changes).
+int ragged_layout(bool lengths, int B, int Hq, int Hkv, int Skv, int D, size_t workspace_bytes, int* splits) {
+  if (!lengths) return 0;
+  const int r = decode_ragged_splits(B, Hq, Hkv, Skv, D, *splits);
+  if (r == *splits || decode_workspace_bytes(B, Hq, D, r) > workspace_bytes) return 0;
+  const int equal = *splits;
+  *splits = r;
+  return equal;
+}
+}  // namespace
 }  // namespace loom
 
 extern "C" {
@@ -207,6 +224,7 @@ loom_status loom_attn_decode(const void* q, const void* k_cache, const void* v_c
   const size_t need = decode_workspace_bytes(B, Hq, D, num_splits);
   if (!workspace || workspace_bytes < need) return LOOM_ERR_WORKSPACE;
   if (!aligned16(workspace)) return LOOM_ERR_MISALIGNED;
+  const int equal_splits = ragged_layout(by_model && seqlens_k, B, Hq, Hkv, Skv, D, workspace_bytes, &num_splits);
   KernelCtl ctl;
   if (!make_ctl(&ctl)) return LOOM_ERR_CUDA;
   const size_t rows = static_cast<size_t>(B) * Hq * num_splits;
@@ -215,7 +233,7 @@ loom_status loom_attn_decode(const void* q, const void* k_cache, const void* v_c
                                              (rows * D * sizeof(float) + 255) / 256 * 256);
   DecodeArgs a{q, k_cache, v_cache, seqlens_k, o, lse, o_part, lse_part, B, Hq, Hkv, Skv, D,
                num_splits, scale, g_decode_form, g_decode_cluster, g_decode_stage_plan, by_model, g_decode_tc,
-               decode_sched_word(workspace, B, Hq, D, num_splits)};
+               decode_sched_word(workspace, B, Hq, D, num_splits), equal_splits};
   return launch_decode(a, ctl, static_cast<cudaStream_t>(stream)) == cudaSuccess ? LOOM_OK
                                                                                  : LOOM_ERR_CUDA;
 }
@@ -279,6 +297,7 @@ loom_status loom_attn_decode_paged(const void* q, const void* k_cache, const voi
   const size_t need = decode_workspace_bytes(B, Hq, D, num_splits);
   if (!workspace || workspace_bytes < need) return LOOM_ERR_WORKSPACE;
   if (!aligned16(workspace)) return LOOM_ERR_MISALIGNED;
+  const int equal_splits = ragged_layout(by_model && seqlens_k, B, Hq, Hkv, Skv, D, workspace_bytes, &num_splits);
   KernelCtl ctl;
   if (!make_ctl(&ctl)) return LOOM_ERR_CUDA;
   const size_t rows = static_cast<size_t>(B) * Hq * num_splits;
@@ -287,7 +306,7 @@ loom_status loom_attn_decode_paged(const void* q, const void* k_cache, const voi
                                              (rows * D * sizeof(float) + 255) / 256 * 256);
   DecodeArgs a{q, k_cache, v_cache, seqlens_k, o, lse, o_part, lse_part, B, Hq, Hkv, Skv, D, num_splits, scale,
                g_decode_form, g_decode_cluster, 0, by_model, g_decode_tc,
-               decode_sched_word(workspace, B, Hq, D, num_splits)};
+               decode_sched_word(workspace, B, Hq, D, num_splits), equal_splits};
   PagedKV pk{block_table, num_pages, page_size, max_pages, kv_layout};
   return launch_decode_paged(a, pk, ctl, static_cast<cudaStream_t>(stream)) == cudaSuccess ? LOOM_OK
                                                                                           : LOOM_ERR_CUDA;
