@@ -297,9 +297,10 @@ __global__ void __launch_bounds__(GemmCfg<BN, NS>::THREADS, 1)
 // stages [r k_iters / S, (r + 1) k_iters / S) into its TMEM accumulator with the same
 // loader / MMA roles as above.  The epilogue warps then park the fp32 partial tile in the
 // CTA's own shared memory (over the ring, which is idle by then), rows 128 B-swizzled in
-// 16-byte chunks; after a cluster barrier CTA r sums rows [r 128 / S, (r + 1) 128 / S)
-// over the S partials in the order s = 0 .. S - 1, reading its peers' shared memory,
-// and stores them as bf16.  A second cluster barrier keeps every partial alive until all
+// 16-byte chunks; after a cluster barrier CTA r sums 1/S of the 16-byte chunks of the tile's
+// rows inside C over the S partials in the order s = 0 .. S - 1, reading its peers' shared
+// memory, and stores them as bf16.  (Summing 128 / S rows per CTA whether C has them or not
+// read eight times too much for a decode step's 16 rows, all of it in one CTA's share.)  A second cluster barrier keeps every partial alive until all
 // peers have read it.  The summation order does not depend on timing, so the result is
 // deterministic for a given S.
 template <int BN, bool BK_MAJOR>
@@ -328,6 +329,7 @@ __global__ void __launch_bounds__(GemmCfg<BN>::SPLIT_THREADS, 1)
   const int tile = static_cast<int>(blockIdx.x) / S;
   int tm, tn;
   tile_coords(p, tile, tm, tn);
+  const int valid = min(C::BM, p.M - tm * C::BM);  // rows of C in this tile: only they are summed
   const int k0 = static_cast<int>(static_cast<long long>(p.k_iters) * rank / S);
   const int k1 = static_cast<int>(static_cast<long long>(p.k_iters) * (rank + 1) / S);
 
@@ -413,7 +415,7 @@ __global__ void __launch_bounds__(GemmCfg<BN>::SPLIT_THREADS, 1)
     // ------------------------------------------------------------------ partial tile -> smem
     const int row = warp * 32 + lane;
     const uint32_t prow = sbase + static_cast<uint32_t>(row) * kRowBytes;
-    if (mbar_wait_warp(bar_acc, 0, p.ctl, ab)) {
+    if (mbar_wait_warp(bar_acc, 0, p.ctl, ab) && warp * 32 < valid) {
       tc_fence_after();
       fence_proxy_async_smem();  // the ring's last TMA writes and MMA reads are complete
       const uint32_t src = tmem + (static_cast<uint32_t>(warp * 32) << 16);
@@ -442,11 +444,12 @@ __global__ void __launch_bounds__(GemmCfg<BN>::SPLIT_THREADS, 1)
 
   if (warp < 4 && !ab.raised()) {
     // ------------------------------------------------------------------ reduce rows, store
-    const int rows = C::BM / S;
     constexpr int kChunks = BN / 4;  // 16-byte chunks of a partial row
-    const int r_first = static_cast<int>(rank) * rows;
-    for (int i = threadIdx.x; i < rows * kChunks; i += 128) {
-      const int r = r_first + i / kChunks, j = i % kChunks;
+    const int all = valid * kChunks;  // chunks of C's rows, dealt evenly to the cluster's CTAs
+    const int log_s = __ffs(S) - 1;
+    const int last = (all * (static_cast<int>(rank) + 1)) >> log_s;
+    for (int i = ((all * static_cast<int>(rank)) >> log_s) + static_cast<int>(threadIdx.x); i < last; i += 128) {
+      const int r = i / kChunks, j = i % kChunks;
       const uint32_t off = static_cast<uint32_t>(r) * kRowBytes + ((static_cast<uint32_t>(j) ^ (r & 7)) << 4);
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int s = 0; s < S; ++s) {
@@ -457,7 +460,7 @@ __global__ void __launch_bounds__(GemmCfg<BN>::SPLIT_THREADS, 1)
         acc.w += v.w;
       }
       const int grow = tm * C::BM + r, gcol = tn * BN + j * 4;
-      if (grow < p.M && gcol < p.N) {  // N % 8 == 0: the 4 columns are all inside C
+      if (gcol < p.N) {  // N % 8 == 0: the 4 columns are all inside C
         uint2 w;
         w.x = pack_bf16x2(acc.x, acc.y);
         w.y = pack_bf16x2(acc.z, acc.w);

@@ -122,6 +122,21 @@ def test_split_parity(loom, forced, tile_n, splits, M, K, N):
 
 
 @pytest.mark.parametrize("splits", SPLITS, ids=[f"s{s}" for s in SPLITS])
+@pytest.mark.parametrize("M", [1, 3, 16, 31, 33, 127, 129])
+def test_split_sums_the_rows_of_c_only(loom, forced, splits, M):
+    """Few rows in a tile: the cluster's CTAs share the sums of those rows' 16-byte chunks."""
+    import torch
+    forced(192, splits)
+    K, N = 2048, 392
+    a, b = _inputs(M + splits, M, K, N)
+    guard = torch.full((M + 8, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    c = loom.loom_gemm_bf16(to_dev(a), to_dev(b), guard[:M])
+    loom.loom_attn_check_error()
+    _check(c.float().cpu().numpy().astype(np.float64), oracle.gemm(a, b), K, f"M={M} S={splits}")
+    assert bool((guard[M:] == 7.0).all())
+
+
+@pytest.mark.parametrize("splits", SPLITS, ids=[f"s{s}" for s in SPLITS])
 def test_split_with_idle_ctas(loom, forced, splits):
     """K = 64 is one stage: all but one CTA of each cluster get no stage and add zeros."""
     forced(64, splits)
