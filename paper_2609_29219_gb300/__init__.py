@@ -163,9 +163,46 @@ def capi() -> ctypes.CDLL:
 
 
 # ------------------------------------------------------------------ marshalling helpers
+# A decode step or a small prefill takes the device 5 to 10 us, so what these helpers cost per
+# argument is what such a call costs.  GB300 host, us per call before and after: prefill of 128
+# rows 16.4 -> 10.8, one decode step 15.3 -> 10.8, GEMM of 16 rows 15.0 -> 9.2.  Most of it was
+# torch.cuda.current_stream (2.0; the raw stream 0.1), the outputs' torch.empty (3.7 between
+# two launches; 1.7 by the call below), and the checks, lock and import statement per argument
+# (0.45; 0.3 in one expression).
+_torch_mod = None
+
+
+_empty_strided_cuda = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_mod, _empty_strided_cuda
+    if _torch_mod is None:
+        import torch
+        try:  # what torch's generated code allocates by: no dispatch, on the current device
+            from torch._C._dynamo.guards import _empty_strided_cuda as call
+            if hasattr(torch._C, "_cuda_getDevice"):
+                _empty_strided_cuda = call
+        except ImportError:
+            pass
+        _torch_mod = torch
+    return _torch_mod
+
+
+def _new(shape, strides, dtype, t):
+    """An uninitialised contiguous tensor (strides: its strides) on CUDA tensor t's device."""
+    torch = _torch_mod
+    if _empty_strided_cuda is not None and t.get_device() == torch._C._cuda_getDevice():
+        return _empty_strided_cuda(shape, strides, dtype)
+    return torch.empty(shape, dtype=dtype, device=t.device)
+
+
+def _ptr(t, name, dtype, ndim):
+    """_dev_ptr of a tensor that passes its checks, in one expression (it names what fails)."""
+    if (isinstance(t, _torch_mod.Tensor) and t.is_cuda and t.dtype is dtype and t.dim() == ndim
+            and t.is_contiguous()):
+        return t.data_ptr()
+    return _dev_ptr(t, name, dtype, ndim)
 
 
 def _dev_ptr(t, name, dtype=None, ndim=None):
@@ -183,6 +220,15 @@ def _dev_ptr(t, name, dtype=None, ndim=None):
     return t.data_ptr()
 
 
+def _stream_of(stream, t):
+    """The given stream, or the current one of tensor t's device, as an integer."""
+    if stream is None:
+        raw = getattr(_torch_mod._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return raw(t.get_device())
+    return _stream_ptr(stream, t.device)
+
+
 def _stream_ptr(stream, device):
     torch = _torch()
     if stream is None:
@@ -191,7 +237,7 @@ def _stream_ptr(stream, device):
 
 
 def _check(status: int, where: str):
-    if status != 0:
+    if status:
         raise LoomError(status, where)
 
 
@@ -205,20 +251,20 @@ def loom_attn_fwd(q, k, v, o=None, lse=None, *, causal=False, scale=None, stream
     """
     torch = _torch()
     bf16 = torch.bfloat16
-    qp = _dev_ptr(q, "q", bf16, 4)
-    kp = _dev_ptr(k, "k", bf16, 4)
-    vp_ = _dev_ptr(v, "v", bf16, 4)
+    qp = _ptr(q, "q", bf16, 4)
+    kp = _ptr(k, "k", bf16, 4)
+    vp_ = _ptr(v, "v", bf16, 4)
     B, Hq, Sq, D = q.shape
     Bk, Hkv, Skv, Dk = k.shape
-    if tuple(v.shape) != tuple(k.shape) or Bk != B or Dk != D:
+    if v.shape != k.shape or Bk != B or Dk != D:
         raise ValueError("q/k/v shapes disagree")
     if o is None:
-        o = torch.empty_like(q)
-    if tuple(o.shape) != tuple(q.shape):
+        o = _new((B, Hq, Sq, D), (Hq * Sq * D, Sq * D, D, 1), bf16, q)
+    if o.shape != q.shape:
         raise ValueError("o must have q's shape")
-    op = _dev_ptr(o, "o", bf16, 4)
+    op = _ptr(o, "o", bf16, 4)
     if lse is None and return_lse:
-        lse = torch.empty((B, Hq, Sq), dtype=torch.float32, device=q.device)
+        lse = _new((B, Hq, Sq), (Hq * Sq, Sq, 1), torch.float32, q)
     lp = None
     if lse is not None:
         if tuple(lse.shape) != (B, Hq, Sq):
@@ -226,8 +272,8 @@ def loom_attn_fwd(q, k, v, o=None, lse=None, *, causal=False, scale=None, stream
         lp = _dev_ptr(lse, "lse", torch.float32)
     if scale is None:
         scale = D ** -0.5
-    st = capi().loom_attn_fwd(qp, kp, vp_, op, lp, B, Hq, Hkv, Sq, Skv, D, int(bool(causal)),
-                              float(scale), _stream_ptr(stream, q.device))
+    st = (_lib or capi()).loom_attn_fwd(qp, kp, vp_, op, lp, B, Hq, Hkv, Sq, Skv, D, int(bool(causal)), float(scale),
+                                        _stream_of(stream, q))
     _check(st, "loom_attn_fwd")
     return (o, lse) if (return_lse or lse is not None) else o
 
@@ -244,23 +290,23 @@ def _decode_operands(q, k_cache, v_cache, seqlens_k, o, lse, return_lse):
     """Pointers and sizes of the contiguous decode entry points' tensor arguments."""
     torch = _torch()
     bf16 = torch.bfloat16
-    qp = _dev_ptr(q, "q", bf16, 4)
-    kp = _dev_ptr(k_cache, "k_cache", bf16, 4)
-    vp_ = _dev_ptr(v_cache, "v_cache", bf16, 4)
+    qp = _ptr(q, "q", bf16, 4)
+    kp = _ptr(k_cache, "k_cache", bf16, 4)
+    vp_ = _ptr(v_cache, "v_cache", bf16, 4)
     B, Hq, Sq, D = q.shape
     Bk, Hkv, Skv, Dk = k_cache.shape
-    if Sq != 1 or tuple(v_cache.shape) != tuple(k_cache.shape) or Bk != B or Dk != D:
+    if Sq != 1 or v_cache.shape != k_cache.shape or Bk != B or Dk != D:
         raise ValueError("decode takes q [B,Hq,1,D] and k/v caches [B,Hkv,Skv,D]")
     sp = None
     if seqlens_k is not None:
         if tuple(seqlens_k.shape) != (B,):
             raise ValueError("seqlens_k must be [B]")
-        sp = _dev_ptr(seqlens_k, "seqlens_k", torch.int32)
+        sp = _ptr(seqlens_k, "seqlens_k", torch.int32, 1)
     if o is None:
-        o = torch.empty_like(q)
-    op = _dev_ptr(o, "o", bf16, 4)
+        o = _new((B, Hq, 1, D), (Hq * D, D, D, 1), bf16, q)
+    op = _ptr(o, "o", bf16, 4)
     if lse is None and return_lse:
-        lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device)
+        lse = _new((B, Hq), (Hq, 1), torch.float32, q)
     lp = None
     if lse is not None:
         if lse.numel() != B * Hq:
@@ -285,9 +331,8 @@ def loom_attn_decode(q, k_cache, v_cache, seqlens_k=None, o=None, lse=None, work
     wp = _dev_ptr(workspace, "workspace")
     if scale is None:
         scale = D ** -0.5
-    st = capi().loom_attn_decode(qp, kp, vp_, sp, op, lp, wp, workspace.numel() * workspace.element_size(),
-                                 B, Hq, Hkv, Skv, D, float(scale), int(num_splits),
-                                 _stream_ptr(stream, q.device))
+    st = (_lib or capi()).loom_attn_decode(qp, kp, vp_, sp, op, lp, wp, workspace.numel() * workspace.element_size(),
+                                           B, Hq, Hkv, Skv, D, float(scale), int(num_splits), _stream_of(stream, q))
     _check(st, "loom_attn_decode")
     return (o, lse) if (return_lse or lse is not None) else o
 
@@ -301,8 +346,8 @@ def loom_attn_decode_noalloc(q, k_cache, v_cache, seqlens_k=None, o=None, lse=No
         q, k_cache, v_cache, seqlens_k, o, lse, return_lse)
     if scale is None:
         scale = D ** -0.5
-    st = capi().loom_attn_decode_noalloc(qp, kp, vp_, sp, op, lp, B, Hq, Hkv, Skv, D, float(scale),
-                                         int(num_splits), _stream_ptr(stream, q.device))
+    st = (_lib or capi()).loom_attn_decode_noalloc(qp, kp, vp_, sp, op, lp, B, Hq, Hkv, Skv, D, float(scale),
+                                                   int(num_splits), _stream_of(stream, q))
     _check(st, "loom_attn_decode_noalloc")
     return (o, lse) if (return_lse or lse is not None) else o
 
@@ -314,23 +359,23 @@ def loom_attn_fwd_varlen(q, k, v, cu_seqlens_q, cu_seqlens_k, max_seqlen_q, o=No
     Returns ``o`` ([total_q, Hq, D]) or ``(o, lse)`` with lse [Hq, total_q]."""
     torch = _torch()
     bf16 = torch.bfloat16
-    qp = _dev_ptr(q, "q", bf16, 3)
-    kp = _dev_ptr(k, "k", bf16, 3)
-    vp_ = _dev_ptr(v, "v", bf16, 3)
+    qp = _ptr(q, "q", bf16, 3)
+    kp = _ptr(k, "k", bf16, 3)
+    vp_ = _ptr(v, "v", bf16, 3)
     total_q, Hq, D = q.shape
     total_k, Hkv, Dk = k.shape
-    if tuple(v.shape) != tuple(k.shape) or Dk != D:
+    if v.shape != k.shape or Dk != D:
         raise ValueError("varlen prefill takes q [total_q, Hq, D] and k/v [total_k, Hkv, D]")
-    cqp = _dev_ptr(cu_seqlens_q, "cu_seqlens_q", torch.int32, 1)
-    ckp = _dev_ptr(cu_seqlens_k, "cu_seqlens_k", torch.int32, 1)
+    cqp = _ptr(cu_seqlens_q, "cu_seqlens_q", torch.int32, 1)
+    ckp = _ptr(cu_seqlens_k, "cu_seqlens_k", torch.int32, 1)
     if cu_seqlens_q.numel() != cu_seqlens_k.numel() or cu_seqlens_q.numel() < 2:
         raise ValueError("cu_seqlens_q and cu_seqlens_k must both be [B + 1]")
     B = cu_seqlens_q.numel() - 1
     if o is None:
-        o = torch.empty_like(q)
-    op = _dev_ptr(o, "o", bf16, 3)
+        o = _new((total_q, Hq, D), (Hq * D, D, 1), bf16, q)
+    op = _ptr(o, "o", bf16, 3)
     if lse is None and return_lse:
-        lse = torch.empty((Hq, total_q), dtype=torch.float32, device=q.device)
+        lse = _new((Hq, total_q), (total_q, 1), torch.float32, q)
     lp = None
     if lse is not None:
         if lse.numel() != Hq * total_q:
@@ -338,9 +383,9 @@ def loom_attn_fwd_varlen(q, k, v, cu_seqlens_q, cu_seqlens_k, max_seqlen_q, o=No
         lp = _dev_ptr(lse, "lse", torch.float32)
     if scale is None:
         scale = D ** -0.5
-    st = capi().loom_attn_fwd_varlen(qp, kp, vp_, op, lp, cqp, ckp, B, Hq, Hkv, total_q, total_k,
-                                     int(max_seqlen_q), D, int(bool(causal)), float(scale),
-                                     _stream_ptr(stream, q.device))
+    st = (_lib or capi()).loom_attn_fwd_varlen(qp, kp, vp_, op, lp, cqp, ckp, B, Hq, Hkv, total_q, total_k,
+                                               int(max_seqlen_q), D, int(bool(causal)), float(scale),
+                                               _stream_of(stream, q))
     _check(st, "loom_attn_fwd_varlen")
     return (o, lse) if (return_lse or lse is not None) else o
 
@@ -353,9 +398,9 @@ def loom_attn_decode_paged(q, k_cache, v_cache, block_table, seqlens_k, o=None, 
     ``o`` or ``(o, lse)``."""
     torch = _torch()
     bf16 = torch.bfloat16
-    qp = _dev_ptr(q, "q", bf16, 4)
-    kp = _dev_ptr(k_cache, "k_cache", bf16, 4)
-    vp_ = _dev_ptr(v_cache, "v_cache", bf16, 4)
+    qp = _ptr(q, "q", bf16, 4)
+    kp = _ptr(k_cache, "k_cache", bf16, 4)
+    vp_ = _ptr(v_cache, "v_cache", bf16, 4)
     B, Hq, Sq, D = q.shape
     if layout not in ("nhd", "hnd"):
         raise ValueError("layout is 'nhd' or 'hnd'")
@@ -363,20 +408,20 @@ def loom_attn_decode_paged(q, k_cache, v_cache, block_table, seqlens_k, o=None, 
         num_pages, page_size, Hkv, Dk = k_cache.shape
     else:
         num_pages, Hkv, page_size, Dk = k_cache.shape
-    if Sq != 1 or tuple(v_cache.shape) != tuple(k_cache.shape) or Dk != D:
+    if Sq != 1 or v_cache.shape != k_cache.shape or Dk != D:
         raise ValueError("paged decode takes q [B,Hq,1,D] and two caches of one shape")
     if block_table.dim() != 2 or block_table.shape[0] != B:
         raise ValueError("block_table must be [B, max_pages]")
     max_pages = block_table.shape[1]
-    tp = _dev_ptr(block_table, "block_table", torch.int32, 2)
+    tp = _ptr(block_table, "block_table", torch.int32, 2)
     if tuple(seqlens_k.shape) != (B,):
         raise ValueError("seqlens_k must be [B]")
-    sp = _dev_ptr(seqlens_k, "seqlens_k", torch.int32)
+    sp = _ptr(seqlens_k, "seqlens_k", torch.int32, 1)
     if o is None:
-        o = torch.empty_like(q)
-    op = _dev_ptr(o, "o", bf16, 4)
+        o = _new((B, Hq, 1, D), (Hq * D, D, D, 1), bf16, q)
+    op = _ptr(o, "o", bf16, 4)
     if lse is None and return_lse:
-        lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device)
+        lse = _new((B, Hq), (Hq, 1), torch.float32, q)
     lp = None
     if lse is not None:
         if lse.numel() != B * Hq:
@@ -389,10 +434,9 @@ def loom_attn_decode_paged(q, k_cache, v_cache, block_table, seqlens_k, o=None, 
     wp = _dev_ptr(workspace, "workspace")
     if scale is None:
         scale = D ** -0.5
-    st = capi().loom_attn_decode_paged(qp, kp, vp_, tp, sp, op, lp, wp, workspace.numel() * workspace.element_size(),
-                                       B, Hq, Hkv, num_pages, page_size, max_pages, 0 if layout == "nhd" else 1,
-                                       D, float(scale),
-                                       int(num_splits), _stream_ptr(stream, q.device))
+    st = (_lib or capi()).loom_attn_decode_paged(
+        qp, kp, vp_, tp, sp, op, lp, wp, workspace.numel() * workspace.element_size(), B, Hq, Hkv, num_pages, page_size,
+        max_pages, 0 if layout == "nhd" else 1, D, float(scale), int(num_splits), _stream_of(stream, q))
     _check(st, "loom_attn_decode_paged")
     return (o, lse) if (return_lse or lse is not None) else o
 
@@ -445,8 +489,8 @@ def loom_gemm_bf16(a, b, c=None, *, stream=None, b_transposed=False):
     ([M, N] bf16, allocated if None)."""
     torch = _torch()
     bf16 = torch.bfloat16
-    ap = _dev_ptr(a, "a", bf16, 2)
-    bp = _dev_ptr(b, "b", bf16, 2)
+    ap = _ptr(a, "a", bf16, 2)
+    bp = _ptr(b, "b", bf16, 2)
     M, K = a.shape
     if b_transposed:
         N, K2 = b.shape
@@ -455,12 +499,13 @@ def loom_gemm_bf16(a, b, c=None, *, stream=None, b_transposed=False):
     if K2 != K:
         raise ValueError(f"a is [M, {K}] but b has {K2} along K")
     if c is None:
-        c = torch.empty((M, N), dtype=bf16, device=a.device)
-    cp = _dev_ptr(c, "c", bf16, 2)
+        c = _new((M, N), (N, 1), bf16, a)
+    cp = _ptr(c, "c", bf16, 2)
     if tuple(c.shape) != (M, N):
         raise ValueError("c must be [M, N]")
-    fn = capi().loom_gemm_bf16_bt if b_transposed else capi().loom_gemm_bf16
-    _check(fn(ap, bp, cp, M, N, K, _stream_ptr(stream, a.device)), "loom_gemm_bf16")
+    lib = _lib or capi()
+    fn = lib.loom_gemm_bf16_bt if b_transposed else lib.loom_gemm_bf16
+    _check(fn(ap, bp, cp, M, N, K, _stream_of(stream, a)), "loom_gemm_bf16")
     return c
 
 
