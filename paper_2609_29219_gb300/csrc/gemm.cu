@@ -67,6 +67,7 @@ struct GemmParams {
   int splits;  // split-K kernel: CTAs per cluster (= per tile)
   int group;   // tile rows per group of the tile order
   int k_alt;   // CTA-pair kernel: 1 walks K backwards in every other round of tiles
+  int a_rows;    // rows of A in a stage's box: 128, fewer when C has fewer (see make_params)
   int b_blocks;  // B [K, N]: 1 when tm_b views B as 64-column blocks (a stage's B in one box)
   int narrow_from;  // CTA-pair kernel: units from here on are 256 x 128 halves of the last tiles
   int n_units;      // CTA-pair kernel: work units (whole tiles, then the narrow halves)
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(GemmCfg<BN, NS>::THREADS, 1)
             continue;
           }
           const uint32_t dst = sbase + s * C::STAGE_BYTES;
-          mbar_expect_tx(bar_full + 8 * s, C::STAGE_BYTES);
+          mbar_expect_tx(bar_full + 8 * s, C::STAGE_BYTES - C::A_BYTES + p.a_rows * 128);
           tma_load_3d(dst, &tm_a, ks * C::BK, tm * C::BM, 0, bar_full + 8 * s);
           if constexpr (BK_MAJOR) {  // BN rows of B [N, K], 64 K-columns: one box
             tma_load_3d(dst + C::A_BYTES, &tm_b, ks * C::BK, tn * BN, 0, bar_full + 8 * s);
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(GemmCfg<BN>::SPLIT_THREADS, 1)
           continue;
         }
         const uint32_t dst = sbase + s * C::STAGE_BYTES;
-        mbar_expect_tx(bar_full + 8 * s, C::STAGE_BYTES);
+        mbar_expect_tx(bar_full + 8 * s, C::STAGE_BYTES - C::A_BYTES + p.a_rows * 128);
         tma_load_3d(dst, &tm_a, ks * C::BK, tm * C::BM, 0, bar_full + 8 * s);
         if constexpr (BK_MAJOR) {
           tma_load_3d(dst + C::A_BYTES, &tm_b, ks * C::BK, tn * BN, 0, bar_full + 8 * s);
@@ -822,6 +823,11 @@ GemmParams make_params(const GemmArgs& a, const KernelCtl& ctl, int bn, int spli
   p.k_iters = (a.K + 63) / 64;
   p.splits = splits;
   p.group = a.group > 0 ? a.group : 8;
+  // Below 128 rows the box of A is as high as C, in whole swizzle periods, not 128 rows that
+  // the copy engine fills with zeros: the MMA rows past it multiply what the slot held, which
+  // only reaches accumulator rows that C does not have.  GB300, us: M 1 N 6144 K 4096 11.0 ->
+  // 7.7, M 16 8.3 -> 8.1, M 1 N 4096 K 4096 12.6 -> 7.2 (7.4 with B [K, N]), M 96 unchanged.
+  p.a_rows = a.M < 128 ? (a.M + 7) / 8 * 8 : 128;
   p.k_alt = 0;
   p.b_blocks = 0;
   p.narrow_from = 0x7fffffff;
@@ -848,8 +854,8 @@ cudaError_t launch_bn(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stre
   if (!set_smem_attr<BN, NS>(reinterpret_cast<const void*>(gemm_kernel<BN, BKM, NS>), configured, dev))
     return cudaErrorInvalidValue;
   CUtensorMap ma, mb, mc;
-  if (!make_maps(a, C::BM, BN, &ma, &mb, &mc)) return cudaErrorInvalidValue;
   GemmParams p = make_params(a, ctl, BN, 1);
+  if (!make_maps(a, p.a_rows, BN, &ma, &mb, &mc)) return cudaErrorInvalidValue;
   use_b_blocks(a, C::NB, &mb, &p);
   const long long tiles = static_cast<long long>(p.tiles_m) * p.tiles_n;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -939,8 +945,8 @@ template <int BN, bool BKM>
 cudaError_t launch_splitk(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stream, int dev, int S) {
   if (!prepare_splitk<BN, BKM>(dev)) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
-  if (!make_maps(a, GemmCfg<BN>::BM, BN, &ma, &mb, nullptr)) return cudaErrorInvalidValue;
   GemmParams p = make_params(a, ctl, BN, S);
+  if (!make_maps(a, p.a_rows, BN, &ma, &mb, nullptr)) return cudaErrorInvalidValue;
   use_b_blocks(a, GemmCfg<BN>::NB, &mb, &p);
   const long long ctas = static_cast<long long>(p.tiles_m) * p.tiles_n * S;
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
