@@ -2238,19 +2238,22 @@ cudaError_t launch_design(Kernel kernel, int rows_per_item, const FwdArgs& a, co
       cfg.blockDim = dim3(C::THREADS);
       cfg.dynamicSmemBytes = C::BYTES;
       cfg.stream = stream;
-      cudaLaunchAttribute attr[1];
+      cudaLaunchAttribute attr[2];
       attr[0].id = cudaLaunchAttributeClusterDimension;
       attr[0].val.clusterDim.x = static_cast<unsigned>(S);
       attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
-      cfg.numAttrs = 1;
+      cfg.numAttrs = 2;
       auto split_kernel = S == 2   ? attn_fwd_kernel<D, false, 0, 2>
                           : S == 4 ? attn_fwd_kernel<D, false, 0, 4>
                                    : attn_fwd_kernel<D, false, 0, 8>;
       return cudaLaunchKernelEx(&cfg, split_kernel, mq, mk, mv, mo, p);
     }
   }
-  return launch_dependent(!a.causal, kernel, workers, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
+  // (a causal launch of one round has no order of CTAs to keep: see launch_dependent)
+  return launch_dependent(!a.causal || items <= sms, kernel, workers, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
 }
 
 // Ring depths compiled for the block-size ablation of the two-tile design (the model's
@@ -2297,8 +2300,13 @@ cudaError_t launch_fwd_d(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t st
   }
   static PerDeviceOnce configured_one;
   constexpr int kRows = FwdCfg<D>::NQT * FwdCfg<D>::BM;
-  const long long last = (static_cast<long long>(a.Sq) << fwd_pack_log2(a.Hq / a.Hkv, a.Sq)) % kRows;
-  if (last > 0 && last <= FwdCfg<D>::BM)  // a plane's last item has one query tile
+  // A plane's last item may have one query tile.  Running it as one pays off while the plane
+  // has few items (B8 H16/2 S300 causal: 15.2 -> 10.3 us); with many, the half item saved is
+  // less than the 2 % that the kernel with ONE is slower (B16 H8/1 S2000, 63 items: 178 us
+  // with the tile past the end computed, 185 without).  A causal last item is its longest.
+  const long long rows = static_cast<long long>(a.Sq) << fwd_pack_log2(a.Hq / a.Hkv, a.Sq);
+  const long long last = rows % kRows;
+  if (last > 0 && last <= FwdCfg<D>::BM && rows <= (a.causal ? 24 : 12) * static_cast<long long>(kRows))
     return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D>, kRows, a, ctl, stream, configured_one);
   return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D, false, 0, 0, false>, FwdCfg<D>::NQT * FwdCfg<D>::BM, a, ctl, stream,
                                      configured2);

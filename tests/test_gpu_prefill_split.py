@@ -29,6 +29,8 @@ SHAPES = [
     (1, 8, 1, 300, 2049, 64, True), (1, 8, 8, 2048, 2048, 128, True), (1, 4, 4, 1500, 1500, 64, True),
     (1, 6, 1, 130, 2300, 128, False), (2, 4, 4, 129, 5000, 64, False), (1, 32, 1, 65, 1025, 128, True),
     (1, 12, 1, 129, 4096, 64, True), (3, 16, 4, 257, 2600, 128, False),
+    # a last item of one tile among few of its plane, and among many (computed as two)
+    (9, 16, 2, 300, 300, 64, True), (2, 4, 4, 3400, 300, 128, False),
 ]
 
 
