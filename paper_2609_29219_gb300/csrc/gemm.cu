@@ -449,23 +449,43 @@ __global__ void __launch_bounds__(GemmCfg<BN>::SPLIT_THREADS, 1)
     const int all = valid * kChunks;  // chunks of C's rows, dealt evenly to the cluster's CTAs
     const int log_s = __ffs(S) - 1;
     const int last = (all * (static_cast<int>(rank) + 1)) >> log_s;
-    for (int i = ((all * static_cast<int>(rank)) >> log_s) + static_cast<int>(threadIdx.x); i < last; i += 128) {
-      const int r = i / kChunks, j = i % kChunks;
-      const uint32_t off = static_cast<uint32_t>(r) * kRowBytes + ((static_cast<uint32_t>(j) ^ (r & 7)) << 4);
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int s = 0; s < S; ++s) {
-        const float4 v = ld_dsmem_f4(map_shared_rank(sbase + off, static_cast<uint32_t>(s)));
-        acc.x += v.x;
-        acc.y += v.y;
-        acc.z += v.z;
-        acc.w += v.w;
+    // kBatch chunks per thread at a time: a remote read's latency, not its bytes, is what a
+    // chunk on its own waits for
+    constexpr int kBatch = 4;
+    for (int i0 = ((all * static_cast<int>(rank)) >> log_s) + static_cast<int>(threadIdx.x); i0 < last;
+         i0 += 128 * kBatch) {
+      float4 acc[kBatch];
+      uint32_t off[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int i = min(i0 + 128 * u, last - 1);  // (past the end: read again, not stored)
+        const int r = i / kChunks, j = i % kChunks;
+        off[u] = sbase + static_cast<uint32_t>(r) * kRowBytes + ((static_cast<uint32_t>(j) ^ (r & 7)) << 4);
+        acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      const int grow = tm * C::BM + r, gcol = tn * BN + j * 4;
-      if (gcol < p.N) {  // N % 8 == 0: the 4 columns are all inside C
-        uint2 w;
-        w.x = pack_bf16x2(acc.x, acc.y);
-        w.y = pack_bf16x2(acc.z, acc.w);
-        *reinterpret_cast<uint2*>(p.c + static_cast<size_t>(grow) * p.N + gcol) = w;
+#pragma unroll 2
+      for (int s = 0; s < S; ++s) {
+        float4 v[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) v[u] = ld_dsmem_f4(map_shared_rank(off[u], static_cast<uint32_t>(s)));
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          acc[u].x += v[u].x;
+          acc[u].y += v[u].y;
+          acc[u].z += v[u].z;
+          acc[u].w += v[u].w;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int i = i0 + 128 * u;
+        const int grow = tm * C::BM + i / kChunks, gcol = tn * BN + (i % kChunks) * 4;
+        if (i < last && gcol < p.N) {  // N % 8 == 0: the 4 columns are all inside C
+          uint2 w;
+          w.x = pack_bf16x2(acc[u].x, acc[u].y);
+          w.y = pack_bf16x2(acc[u].z, acc[u].w);
+          *reinterpret_cast<uint2*>(p.c + static_cast<size_t>(grow) * p.N + gcol) = w;
+        }
       }
     }
   }
