@@ -286,7 +286,7 @@ __device__ __forceinline__ Item make_item_t(const FwdParams& p, const SeqCursor&
     it.kb = p.cu_k[cur.b];
     it.skv = p.cu_k[cur.b + 1] - it.kb;
     it.q0 = pos * (C::NQT * C::BM);
-    const bool two = it.q0 + C::BM < it.sq;
+    const bool two = !ONE || it.q0 + C::BM < it.sq;
     it.q1 = two ? it.q0 + C::BM : it.q0;
     const int off = it.skv - it.sq;
     int n_kv0 = it.skv, n_kv1 = it.skv;
@@ -2041,7 +2041,7 @@ cudaError_t launch_dependent(bool dependent, Kernel kernel, int grid, int thread
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <int D>
+template <int D, bool ONE>
 cudaError_t launch_varlen_d(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaStream_t stream) {
   using C = FwdCfg<D>;
   static PerDeviceOnce configured;
@@ -2054,7 +2054,7 @@ cudaError_t launch_varlen_d(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaSt
   int dev = 0;
   cudaGetDevice(&dev);
   if (!configured.run(dev, [] {
-        return cudaFuncSetAttribute(attn_fwd_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(attn_fwd_kernel<D, true, 0, 0, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     C::BYTES) == cudaSuccess;
       }))
     return cudaErrorInvalidValue;
@@ -2079,7 +2079,7 @@ cudaError_t launch_varlen_d(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaSt
   constexpr int kRows = C::NQT * C::BM;
   const long long bound = static_cast<long long>(a.B) * a.Hq * ((a.max_seqlen_q + kRows - 1) / kRows);
   const int grid = static_cast<int>(bound > 0 && bound < sms ? bound : sms);
-  return launch_dependent(false, attn_fwd_kernel<D, true>, grid, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
+  return launch_dependent(false, attn_fwd_kernel<D, true, 0, 0, ONE>, grid, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
 }
 
 // Query heads of one kv head packed into a plane of the two-tile design (as a power of two):
@@ -2320,8 +2320,13 @@ cudaError_t launch_fwd(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t stre
 }
 
 cudaError_t launch_fwd_varlen(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaStream_t stream) {
-  if (a.D == 128) return launch_varlen_d<128>(a, ctl, stream);
-  return launch_varlen_d<64>(a, ctl, stream);
+  // Without a causal mask and with 8 query-tile pairs or more per sequence on average, the half
+  // item that a one-tile item saves is less than what its kernel costs (8 sequences of 1024 to
+  // 4096, H64/16 D64: 1022 us with ONE, 1005 without; H32/8 D128: 614 and 602).  A causal
+  // sequence's last item is its longest (12 of 1500 to 6000, H32/8: 1032 with, 1046 without).
+  if (!a.causal && a.total_q >= 8ll * 256 * a.B)
+    return a.D == 128 ? launch_varlen_d<128, false>(a, ctl, stream) : launch_varlen_d<64, false>(a, ctl, stream);
+  return a.D == 128 ? launch_varlen_d<128, true>(a, ctl, stream) : launch_varlen_d<64, true>(a, ctl, stream);
 }
 
 }  // namespace loom
