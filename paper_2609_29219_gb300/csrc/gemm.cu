@@ -38,7 +38,7 @@ template <int BN, int NS = 0>
 struct GemmCfg {
   static constexpr model::GemmPlan kPlan = model::gemm_plan_variant(BN);
   static_assert(kPlan.feasible, "no feasible GEMM plan for this tile width");
-  static constexpr int BM = 128, BK = 64;
+  static constexpr int BM = 128, BK = 64, A_ROWS = BM;
   static constexpr int NSTAGE = NS ? NS : kPlan.stages;
   static constexpr int THREADS = 320;                       // 8 epilogue warps, loader, MMA
   static constexpr int SPLIT_THREADS = 192;                 // split-K: 4 epilogue warps, loader, MMA
@@ -58,6 +58,33 @@ struct GemmCfg {
                                         : 2 * BN <= 256 ? 256 : 512;
   static_assert(STG_WARP * 8 == model::kGemmStagingBytes, "staging layout matches the model");
   static_assert(BYTES <= 227 * 1024, "shared memory budget");
+};
+
+// The split-K kernel for at most 32 rows of C: a stage's A tile is 4 KB (the MMA's other 96
+// rows read on into the stage's B tile and past it, in this CTA's shared memory, and only
+// reach accumulator rows that C does not have), and the ring is half an SM's shared memory,
+// so that two CTAs share an SM: the next launch's CTAs, or the other half of the splits, are
+// there when this one's first bytes are still on their way.  It needs two CTAs on many of the
+// SMs to keep as many bytes in flight as one of the large ring does (kSkinnyMinCtas).
+constexpr int kSkinnyRows = 32, kSkinnyMinCtas = 176;
+template <int BN>
+struct GemmSkinnyCfg {
+  static constexpr int BM = 128, BK = 64, A_ROWS = kSkinnyRows;
+  static constexpr int SPLIT_THREADS = 192;
+  static constexpr int NB = BN / 64;
+  static constexpr uint32_t A_BYTES = A_ROWS * BK * 2;
+  static constexpr uint32_t B_BOX_BYTES = BK * 64 * 2;
+  static constexpr uint32_t STAGE_BYTES = A_BYTES + NB * B_BOX_BYTES;
+  static constexpr uint32_t PAST_BYTES = STAGE_BYTES < BM * BK * 2 ? BM * BK * 2 - STAGE_BYTES : 0;
+  static constexpr int NSTAGE = (112 * 1024 - static_cast<int>(PAST_BYTES)) / static_cast<int>(STAGE_BYTES + 512);
+  static constexpr uint32_t STG_OFF = NSTAGE * STAGE_BYTES;
+  static constexpr uint32_t BAR_OFF = STG_OFF + PAST_BYTES;
+  static constexpr int NBAR = 2 * NSTAGE + 5;
+  static constexpr uint32_t TMEM_PTR_OFF = BAR_OFF + NBAR * 8;
+  static constexpr uint32_t ABORT_OFF = TMEM_PTR_OFF + 8;
+  static constexpr uint32_t BYTES = ABORT_OFF + 16 + 1024;  // + alignment slack
+  static_assert(STAGE_BYTES % 1024 == 0, "swizzled tiles start on the swizzle period");
+  static_assert(2 * (BYTES + 1024) <= 228 * 1024, "two CTAs per SM");
 };
 
 struct GemmParams {
@@ -304,14 +331,13 @@ __global__ void __launch_bounds__(GemmCfg<BN, NS>::THREADS, 1)
 // read eight times too much for a decode step's 16 rows, all of it in one CTA's share.)  A second cluster barrier keeps every partial alive until all
 // peers have read it.  The summation order does not depend on timing, so the result is
 // deterministic for a given S.
-template <int BN, bool BK_MAJOR>
-__global__ void __launch_bounds__(GemmCfg<BN>::SPLIT_THREADS, 1)
+template <int BN, bool BK_MAJOR, class C = GemmCfg<BN>>
+__global__ void __launch_bounds__(C::SPLIT_THREADS, 1)
     gemm_splitk_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                        const GemmParams p) {
-  using C = GemmCfg<BN>;
   constexpr uint32_t kCols = BN <= 64 ? 64 : BN <= 128 ? 128 : 256;  // one accumulator
   constexpr uint32_t kRowBytes = BN * 4;                                // fp32 partial row
-  static_assert(C::BM * kRowBytes <= C::STG_OFF, "the partial tile fits in the ring");
+  static_assert(C::A_ROWS * kRowBytes <= C::STG_OFF, "the partial tile fits in the ring");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_base = smem_u32(smem_raw);
   const uint32_t sbase = (raw_base + 1023u) & ~1023u;
@@ -894,13 +920,13 @@ cudaError_t launch_bn(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stre
   return cudaLaunchKernelEx(&cfg, gemm_kernel<BN, BKM, NS>, ma, mb, mc, p);
 }
 
-template <int BN>
+template <int BN, class C = GemmCfg<BN>>
 cudaLaunchConfig_t splitk_config(int grid, int S, cudaStream_t stream, cudaLaunchAttribute* attr,
                                  bool dependent = false) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
-  cfg.blockDim = dim3(GemmCfg<BN>::SPLIT_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = GemmCfg<BN>::BYTES;
+  cfg.blockDim = dim3(C::SPLIT_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = C::BYTES;
   cfg.stream = stream;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(S);
@@ -916,11 +942,14 @@ cudaLaunchConfig_t splitk_config(int grid, int S, cudaStream_t stream, cudaLaunc
   return cfg;
 }
 
-template <int BN, bool BKM>
+template <int BN, bool BKM, class C = GemmCfg<BN>>
 bool prepare_splitk(int dev) {
   static PerDeviceOnce configured, nonportable;
-  const void* fn = reinterpret_cast<const void*>(gemm_splitk_kernel<BN, BKM>);
-  if (!set_smem_attr<BN>(fn, configured, dev)) return false;
+  const void* fn = reinterpret_cast<const void*>(gemm_splitk_kernel<BN, BKM, C>);
+  if (!configured.run(dev, [fn] {
+        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES) == cudaSuccess;
+      }))
+    return false;
   return nonportable.run(dev, [fn] {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
   });
@@ -961,9 +990,9 @@ int splitk_slots_any(int dev, int bn, int S) {
   }
 }
 
-template <int BN, bool BKM>
-cudaError_t launch_splitk(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stream, int dev, int S) {
-  if (!prepare_splitk<BN, BKM>(dev)) return cudaErrorInvalidValue;
+template <int BN, bool BKM, class C>
+cudaError_t launch_splitk_cfg(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stream, int dev, int S) {
+  if (!prepare_splitk<BN, BKM, C>(dev)) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
   GemmParams p = make_params(a, ctl, BN, S);
   if (!make_maps(a, p.a_rows, BN, &ma, &mb, nullptr)) return cudaErrorInvalidValue;
@@ -971,8 +1000,17 @@ cudaError_t launch_splitk(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t 
   const long long ctas = static_cast<long long>(p.tiles_m) * p.tiles_n * S;
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg = splitk_config<BN>(static_cast<int>(ctas), S, stream, attr, true);
-  return cudaLaunchKernelEx(&cfg, gemm_splitk_kernel<BN, BKM>, ma, mb, p);
+  cudaLaunchConfig_t cfg = splitk_config<BN, C>(static_cast<int>(ctas), S, stream, attr, true);
+  return cudaLaunchKernelEx(&cfg, gemm_splitk_kernel<BN, BKM, C>, ma, mb, p);
+}
+
+template <int BN, bool BKM>
+cudaError_t launch_splitk(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stream, int dev, int S) {
+  if constexpr (BN == 128) {
+    if (a.M <= kSkinnyRows && static_cast<long long>((a.N + BN - 1) / BN) * S >= kSkinnyMinCtas)
+      return launch_splitk_cfg<BN, BKM, GemmSkinnyCfg<BN>>(a, ctl, stream, dev, S);
+  }
+  return launch_splitk_cfg<BN, BKM, GemmCfg<BN>>(a, ctl, stream, dev, S);
 }
 
 template <bool BKM, int NS = 6>
@@ -1106,6 +1144,19 @@ cudaError_t launch_choice(const GemmArgs& a, const GemmChoice& c, const KernelCt
   }
 }
 
+// Splits of the split-K kernel for at most 32 rows over 128-wide tiles: the most that two CTAs
+// per SM hold, of 16 K stages or more each; 0 where that leaves fewer than kSkinnyMinCtas,
+// and the model's choice with the large ring is as fast.  GB300, weights read from HBM, us,
+// the model's choice / this: M 16 N 6144 K 4096 13.1 / 12.4, M 16 N 16384 K 4096 27.3 / 26.1,
+// M 32 N 12288 K 4096 22.3 / 20.7, M 3 N 5600 K 11432 26.5 / 25.5; not taken: M 1 N 4096 K 4096
+// 9.0 / 9.2, M 8 9.0 / 9.9.
+int skinny_splits(int N, int K, int sms) {
+  const long long tiles = (N + 127) / 128, stages = (K + 63) / 64;
+  for (int S = 16; S >= 2; S /= 2)
+    if (tiles * S <= 2ll * sms && stages >= 16ll * S) return tiles * S >= kSkinnyMinCtas ? S : 0;
+  return 0;
+}
+
 bool device_sms(int* dev, int* sms) {
   if (cudaGetDevice(dev) != cudaSuccess) return false;
   return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev) == cudaSuccess && *sms > 0;
@@ -1116,6 +1167,10 @@ bool device_sms(int* dev, int* sms) {
 GemmChoice gemm_choice(int M, int N, int K, GemmChoice forced) {
   int dev = 0, sms = 0;
   if (!device_sms(&dev, &sms)) return {0, 0};
+  if (forced.tile_n == 0 && forced.splits == 0 && forced.pair == 0 && M <= kSkinnyRows) {
+    const int S = skinny_splits(N, K, sms);
+    if (S > 0) return {128, S, 0};
+  }
   const model::GemmChoiceModel c = model::gemm_choose(
       M, N, K, sms, [dev](int bn, int S) { return splitk_slots_any(dev, bn, S); }, model::kGb300, forced.tile_n,
       forced.splits, forced.pair >= 0 ? pair_slots(dev) : 0, forced.pair);

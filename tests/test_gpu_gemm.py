@@ -136,6 +136,20 @@ def test_split_sums_the_rows_of_c_only(loom, forced, splits, M):
     assert bool((guard[M:] == 7.0).all())
 
 
+@pytest.mark.parametrize("M", [1, 8, 17, 32, 33])
+@pytest.mark.parametrize("N,K", [(6144, 4096), (11264, 2056), (22520, 1024)])
+def test_skinny(loom, M, N, K):
+    """At most 32 rows: the split-K kernel with the small ring (two CTAs per SM) where enough
+    tiles and K stages exist; 33 rows and the shapes past its rule run the other kernels."""
+    import torch
+    a, b = _inputs(M + K, M, K, N)
+    c_ref = oracle.gemm(a, b)
+    _check(_run(loom, a, b), c_ref, K, f"skinny M={M} N={N} K={K}")
+    c = loom.loom_gemm_bf16(to_dev(a), to_dev(b).t().contiguous(), b_transposed=True)
+    loom.loom_attn_check_error()
+    _check(c.float().cpu().numpy().astype(np.float64), c_ref, K, f"skinny M={M} N={N} K={K} transposed")
+
+
 @pytest.mark.parametrize("splits", SPLITS, ids=[f"s{s}" for s in SPLITS])
 def test_split_with_idle_ctas(loom, forced, splits):
     """K = 64 is one stage: all but one CTA of each cluster get no stage and add zeros."""
