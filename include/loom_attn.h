@@ -355,7 +355,8 @@ void loom_debug_prefill_design(int design);
  * constant) when that value is not compiled:
  * loom_debug_prefill_slots: the two-tile prefill's K/V ring depth for head dimension D
  *   (compiled beside the model's 3 at D = 128: 2; beside 10 at D = 64: 3, 6, 9; deeper
- *   rings do not fit in shared memory).  0 restores the model's.
+ *   rings do not fit in shared memory).  0 restores the model's, which at D = 128 runs with
+ *   one slot more, in the memory that the query tiles' shared O staging leaves.
  * loom_debug_decode_stage_plan: the decode split kernel's keys per stage, ring stages and
  *   CTAs per SM (contiguous cache, D = 128, 4 query heads per kv head, split + merge form;
  *   compiled: 32x2x2, 32x3x2, 32x4x2, 64x2x2, 64x4x1, 128x2x1, 128x3x1 beside the model's

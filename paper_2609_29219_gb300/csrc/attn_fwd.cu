@@ -6,8 +6,10 @@
 // counted circular buffers is the virtual-buffer protocol of Sec. 2.3, and the tile and
 // stage constants come from the latency model of Sec. 2.6 (Eq. 6-9, in model.h).
 //
-// One CTA owns NQT = 2 query tiles of BM = 128 rows (tile 0 and tile 1) of one
-// (batch, query head) and walks the key/value sequence in tiles of BN = 128 rows:
+// One CTA owns NQT = 2 query tiles of BM = 128 rows (tile 0 and tile 1) of one plane -- one
+// (batch, query head), or a power of two of the heads of one kv head, whose rows of a query
+// follow one another -- and walks the key/value sequence in tiles of BN = 128 rows.  Launches
+// with few such items give each to a cluster of CTAs that share its keys (split_epilogue).
 //
 //   warp 8 (loader, 1 thread)   Q0, Q1 once; then K_0, V_0, K_1, V_1, ... into an
 //                               NSLOT-deep ring of 128B-swizzled shared-memory slots
@@ -2018,9 +2020,9 @@ bool make_map_packed(CUtensorMap* map, const void* base, int D, int Sq, int plan
 // kernels wait for that kernel (griddepcontrol.wait) after their set-up and before any
 // global access, which costs nothing when they were launched plainly.  Non-causal launches
 // take it (their set-up overlaps the previous grid's tail: +1.3 % on B4 H32 S2048, +10 %
-// on B1 H32 S1024, back to back); causal ones do not (-4 % on B4 H32 S2048 causal: the
-// early CTAs land on SMs in the order the previous grid frees them, which the causal
-// dealing's L2 blocks do not expect).
+// on B1 H32 S1024, back to back), and so do causal ones of one round (H4 S512 10.9 -> 9.9 us);
+// causal ones of more rounds do not (-4 % on B4 H32 S2048 causal: the early CTAs land on SMs in
+// the order the previous grid frees them, which the causal dealing's L2 blocks do not expect).
 template <class Kernel, class... Args>
 cudaError_t launch_dependent(bool dependent, Kernel kernel, int grid, int threads, uint32_t smem,
                              cudaStream_t stream, Args... args) {
