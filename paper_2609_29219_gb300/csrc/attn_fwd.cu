@@ -633,10 +633,12 @@ __device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars ba
   for (int q = 0; q < S; ++q)
     if (q != rank && !mbar_wait_cluster_warp(bar.rdy + 8 * q, r.par_x, ctl, ab)) return false;
   if (r.active) {
+    // (a CTA without tiles of the row sends no O; it says so by a negative sum)
+    const float l_mine = r.has_tiles ? r.l : -1.f;
 #pragma unroll
     for (int q = 0; q < S; ++q) {
       const uint32_t mine = static_cast<uint32_t>(rank < q ? rank : rank - (rank > q)) * kSrc;  // my place in CTA q
-      if (q != rank) st_dsmem_f2(map_shared_rank(partial_at<C>(sbase, mine + kO + rb * 8), q), r.m, r.l);
+      if (q != rank) st_dsmem_f2(map_shared_rank(partial_at<C>(sbase, mine + kO + rb * 8), q), r.m, l_mine);
     }
     if (r.has_tiles) {
 #pragma unroll
@@ -663,12 +665,14 @@ __device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars ba
     // the S partials' weights, in rank order
     float w[S], l = 0.f, M = r.m;
     float2 ml[S];
-    uint32_t src[S];  // source s's place
+    uint32_t src[S];    // source s's place
+    uint32_t sent = 0;  // bit s: source s has sent an O
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       src[s] = static_cast<uint32_t>(s < rank ? s : s - (s > rank)) * kSrc;
-      ml[s] = s == rank ? make_float2(r.m, r.l) : ld_shared_f2(partial_at<C>(sbase, src[s] + kO + rb * 8));
+      ml[s] = s == rank ? make_float2(r.m, l_mine) : ld_shared_f2(partial_at<C>(sbase, src[s] + kO + rb * 8));
       M = fmaxf(M, ml[s].x);
+      sent |= (ml[s].y < 0.f ? 0u : 1u) << s;  // (a NaN sum is one that was sent)
     }
 #pragma unroll
     for (int s = 0; s < S; ++s) {
@@ -699,7 +703,9 @@ __device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars ba
 #pragma unroll
             for (int i = 0; i < U; ++i) acc[i] = fmaf(w[s], __uint_as_float(own[i]), acc[i]);
           }
-        } else if (w[s] != 0.f) {  // (a CTA without tiles of this row has sent no O)
+        } else if (sent >> s & 1u) {
+          // (also with a weight of 0: O may be NaN, of a NaN score or value, and 0 * NaN stays NaN
+          // as it does where one CTA walks all keys)
           uint4 v[U / 4];
 #pragma unroll
           for (int i = 0; i < U / 4; ++i) 

@@ -68,6 +68,46 @@ def test_extreme_scores_across_shares(loom):
     assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy(), lse_ref, "scores of one share dominate")
 
 
+NAN, INF = 0x7FC0, 0x7F80  # bf16 bits
+
+
+# The shape's clusters: of 2 with a first item whose tile 0 falls to one CTA, of 2, of 8
+@pytest.mark.parametrize("tensor,pos,bits", [
+    ("q", 5, NAN), ("q", -1, NAN), ("k", 0, NAN), ("k", 777, NAN), ("k", -1, NAN), ("k", 300, INF), ("v", 0, NAN),
+    ("v", 900, INF), ("v", -1, NAN)])
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,causal", [
+    (1, 8, 8, 2048, 2048, 128, True), (1, 4, 4, 1500, 1500, 64, True), (1, 8, 1, 300, 2049, 64, False)])
+@pytest.mark.parametrize("steep", [False, True])
+def test_nan_and_infinity(loom, steep, tensor, pos, bits, B, Hq, Hkv, Sq, Skv, D, causal):
+    """NaN and infinity reach the same elements as where one CTA walks all keys of an item.
+    steep: the last keys' scores are so large that the other shares' weights are 0."""
+    q = synth.bf16_normal(6, synth.STREAM_Q, (B, Hq, Sq, D))
+    k = synth.bf16_normal(6, synth.STREAM_K, (B, Hkv, Skv, D))
+    v = synth.bf16_normal(6, synth.STREAM_V, (B, Hkv, Skv, D))
+    if steep:
+        kf = (k.astype(np.uint32) << 16).view(np.float32).copy()
+        kf[:, :, -Skv // 16:] *= 200.0
+        k = synth.f32_to_bf16(kf)
+    {"q": q, "k": k, "v": v}[tensor][0, 0, pos, 3] = bits
+    qd, kd, vd = to_dev(q), to_dev(k), to_dev(v)
+    o, lse = loom.loom_attn_fwd(qd, kd, vd, causal=causal, return_lse=True)
+    loom.loom_debug_prefill_slots(D, 2 if D == 128 else 9)  # a pinned ring depth runs one CTA per item
+    try:
+        o1, lse1 = loom.loom_attn_fwd(qd, kd, vd, causal=causal, return_lse=True)
+    finally:
+        loom.loom_debug_prefill_slots(D, 0)
+    loom.loom_attn_check_error()
+    a, b = o_to_f64(o), o_to_f64(o1)
+    assert not np.isfinite(b).all()
+    assert np.array_equal(np.isnan(a), np.isnan(b)), "elements that are NaN"
+    assert np.array_equal(np.isinf(a), np.isinf(b)), "elements that are infinite"
+    fin = np.isfinite(b)
+    # either side rounds P and O to bf16 (2^-9 each, of at most the largest value)
+    vf = (v.astype(np.uint32) << 16).view(np.float32)
+    assert np.abs(a[fin] - b[fin]).max(initial=0.0) <= 2.0 ** -7 * np.abs(vf[np.isfinite(vf)]).max()
+    assert np.allclose(lse.cpu().numpy(), lse1.cpu().numpy(), rtol=1e-5, atol=1e-4, equal_nan=True)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_timeout_in_a_cluster_is_reported(loom, D):
     """A K/V tile that never arrives in any CTA of a cluster: every wait runs out, the call
