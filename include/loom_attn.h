@@ -63,6 +63,14 @@ loom_status loom_attn_fwd(const void* q, const void* k, const void* v, void* o, 
                           void* stream);
 
 /*
+ * CTAs per thread-block cluster that share a work item (a pair of query tiles) of
+ * loom_attn_fwd with these sizes on the current device: 2, 4 or 8 where the items are few
+ * and their keys many, 1 where each item has a CTA of its own (also with a pinned design or
+ * ring depth, see the debug hooks); 0 on invalid sizes or without a device.
+ */
+int loom_attn_fwd_cluster(int B, int Hq, int Hkv, int Sq, int Skv, int D, int causal);
+
+/*
  * Prefill over a ragged batch packed token-major (the packed-varlen layout; the paper has
  * no counterpart -- irregular grids are outside its Sec. 2.6 scope note).
  *   q             [total_q, Hq, D]   bf16, read

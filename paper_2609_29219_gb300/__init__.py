@@ -31,7 +31,7 @@ __all__ = [
     "loom_attn_decode_form", "loom_decode_max_clusters", "loom_decode_persistent_slots", "loom_debug_decode_form",
     "loom_model_decode_persistent_time_us", "loom_model_decode_tc_time_us", "DECODE_SPLIT_MERGE", "DECODE_PERSISTENT", "DECODE_CLUSTER",
     "loom_debug_prefill_slots", "loom_debug_decode_stage_plan", "loom_debug_gemm_stages",
-    "loom_debug_gemm_order", "loom_debug_decode_tensor_cores",
+    "loom_debug_gemm_order", "loom_debug_decode_tensor_cores", "loom_attn_fwd_cluster",
 ]
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -140,6 +140,8 @@ def capi() -> ctypes.CDLL:
             lib.loom_model_decode_persistent_time_us.restype = ctypes.c_double
             lib.loom_model_decode_tc_time_us.argtypes = [i32] * 7
             lib.loom_model_decode_tc_time_us.restype = ctypes.c_double
+            lib.loom_attn_fwd_cluster.argtypes = [i32] * 7
+            lib.loom_attn_fwd_cluster.restype = i32
             lib.loom_attn_decode_form.argtypes = [i32] * 7 + [ctypes.POINTER(i32)]
             lib.loom_attn_decode_form.restype = i32
             lib.loom_decode_max_clusters.argtypes = [i32, i32, i32]
@@ -552,6 +554,12 @@ def loom_model_decode_time_us(splits, B, Hq, Hkv, Skv, D, num_sms) -> float:
 
 def loom_model_decode_cluster_time_us(splits, cluster, B, Hq, Hkv, Skv, D, clusters) -> float:
     return float(capi().loom_model_decode_cluster_time_us(splits, cluster, B, Hq, Hkv, Skv, D, clusters))
+
+
+def loom_attn_fwd_cluster(B, Hq, Hkv, Sq, Skv, D, causal=False) -> int:
+    """CTAs per cluster that share a work item of ``loom_attn_fwd`` with these sizes (1: none
+    do; 0: invalid sizes or no device)."""
+    return int(capi().loom_attn_fwd_cluster(B, Hq, Hkv, Sq, Skv, D, int(bool(causal))))
 
 
 DECODE_SPLIT_MERGE, DECODE_PERSISTENT, DECODE_CLUSTER = 1, 2, 3

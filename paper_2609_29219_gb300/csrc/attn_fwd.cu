@@ -627,12 +627,19 @@ __device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars ba
     if (!mbar_wait_warp(bar.o, r.par_o, ctl, ab)) return false;
     tc_fence_after();
   }
-  // (also without a tile: no warp may run an item ahead of these barriers' phases)
-  if (!r.active && !r.first && !mbar_wait_warp(bar.xdone, r.par_x ^ 1, ctl, ab)) return false;
-#pragma unroll
-  for (int q = 0; q < S; ++q)
-    if (q != rank && !mbar_wait_cluster_warp(bar.rdy + 8 * q, r.par_x, ctl, ab)) return false;
+  // A wait by parity may neither start a phase early nor miss one.
+  //   xdone: its phase r needs this warp's own arrival, so no warp misses phase r - 1, and by
+  //     waiting for it no warp, with or without the tile, arrives or goes on an item ahead.
+  //   rdy: phase r - 1 is over once xdone's is (the warps of tile 1 have waited for it), and
+  //     phase r + 1 needs the peer's xdone of item r, for which the peer's warp of these rows
+  //     needs this warp's partials.  That holds only for a tile that the item has: a warp
+  //     without it sends nothing and must not wait on rdy at all.
+  //   xf: phase r + 1 needs the peers' rdy of this CTA, and so this CTA's xdone of item r.
+  if (!r.first && !mbar_wait_warp(bar.xdone, r.par_x ^ 1, ctl, ab)) return false;
   if (r.active) {
+#pragma unroll
+    for (int q = 0; q < S; ++q)
+      if (q != rank && !mbar_wait_cluster_warp(bar.rdy + 8 * q, r.par_x, ctl, ab)) return false;
     // (a CTA without tiles of the row sends no O; it says so by a negative sum)
     const float l_mine = r.has_tiles ? r.l : -1.f;
 #pragma unroll
@@ -870,7 +877,14 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
         const Item it = item_of(cur, idx);
         // Q tiles and K slots hold the previous item's partials until every warp has read them
         if (SPLIT && r > 0 && !(ok = mbar_wait(bar_xdone, (r - 1) & 1, p.ctl, ab))) break;
-        if (SPLIT && it.n_tiles == 0) continue;
+        if (SPLIT && it.n_tiles == 0) {
+          // Nothing of this item falls to this CTA: it takes partials at once.  It is this
+          // thread that says so, because xdone's next phase needs the peers' partials: the
+          // wait above would miss a phase if another warp let them come.
+          for (int q = 0; q < S; ++q)
+            if (q != rank) mbar_arrive_cluster(map_shared_rank(bar_rdy + 8 * rank, q));
+          continue;
+        }
         // Q_0 first: tile 0 finishes its S MMAs of the previous item before tile 1 does
         const bool two = !ONE || it.n_tiles0 > 0;
         if (!(ok = load_q(two ? 0 : 1, it))) break;
@@ -952,11 +966,7 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
       for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur, wk, n_wk)) >= 0; ++r) {
         const Item it = item_of(cur, idx);
         const int nt0 = it.n_tiles0, nt = it.n_tiles;
-        if (SPLIT && nt == 0) {  // nothing of this item falls to this CTA: it takes partials at once
-          if (r > 0 && !(ok = mbar_wait_warp(bar_xdone, (r - 1) & 1, p.ctl, ab))) break;
-          if (lane < S && lane != rank) mbar_arrive_cluster(map_shared_rank(bar_rdy + 8 * rank, lane));
-          continue;
-        }
+        if (SPLIT && nt == 0) continue;  // nothing of this item falls to this CTA (see the loader)
         if (!ONE || nt0 > 0) {
           if (!(ok = mbar_wait_warp(bar_q, n0 & 1, p.ctl, ab) && wait_slot(pos))) break;
           tc_fence_after();
@@ -2189,6 +2199,36 @@ int fwd_split(const FwdParams& p, int sms, int dev) {
   return best;
 }
 
+// p, zeroed, with the sizes and work items of a dense launch (planes of 2^lg heads, items of
+// rows_per_item rows); false if there are too many.
+bool set_items(FwdParams& p, const FwdArgs& a, int lg, int rows_per_item) {
+  memset(&p, 0, sizeof(p));
+  p.Hq = a.Hq;
+  p.Hkv = a.Hkv;
+  p.Sq = a.Sq;
+  p.Skv = a.Skv;
+  p.causal = a.causal;
+  p.pack_log2 = lg;
+  p.planes_per_kv = (a.Hq / a.Hkv) >> lg;
+  p.q_rows = a.Sq << lg;
+  p.n_pairs = (p.q_rows + rows_per_item - 1) / rows_per_item;
+  const long long items = static_cast<long long>(p.n_pairs) * ((a.B * a.Hq) >> lg);
+  p.n_items = static_cast<int>(items);
+  return items <= 0x7fffffffLL;
+}
+
+// Cluster size of a dense two-tile launch with these sizes on the current device (0: unknown).
+template <int D>
+int fwd_cluster(const FwdArgs& a) {
+  int dev = 0, sms = 0;
+  FwdParams p;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      !set_items(p, a, fwd_pack_log2(a.Hq / a.Hkv, a.Sq), FwdCfg<D>::NQT * FwdCfg<D>::BM))
+    return 0;
+  return fwd_split<D>(p, sms, dev);
+}
+
 // Launch one design: C is its configuration, rows_per_item the query rows of one work
 // item (C::NQT * C::BM).  PACKED: the two-tile design over planes of packed heads.
 template <int D, class C, bool PACKED = false, class Kernel>
@@ -2210,23 +2250,11 @@ cudaError_t launch_design(Kernel kernel, int rows_per_item, const FwdArgs& a, co
       }))
     return cudaErrorInvalidValue;
   FwdParams p;
-  memset(&p, 0, sizeof(p));
+  if (!set_items(p, a, lg, rows_per_item)) return cudaErrorInvalidConfiguration;
   p.o = static_cast<__nv_bfloat16*>(a.o);
   p.lse = a.lse;
-  p.Hq = a.Hq;
-  p.Hkv = a.Hkv;
-  p.Sq = a.Sq;
-  p.Skv = a.Skv;
-  p.pack_log2 = lg;
-  p.planes_per_kv = (a.Hq / a.Hkv) >> lg;
-  p.q_rows = a.Sq << lg;
-  p.n_pairs = (p.q_rows + rows_per_item - 1) / rows_per_item;
-  p.causal = a.causal;
   p.c = a.scale * kLog2e;
   p.ctl = ctl;
-  const long long items = static_cast<long long>(p.n_pairs) * planes;
-  if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  p.n_items = static_cast<int>(items);
   // persistent: one CTA per SM (shared memory / TMEM admit one), each walking its items
   int sms = 0;
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2236,7 +2264,7 @@ cudaError_t launch_design(Kernel kernel, int rows_per_item, const FwdArgs& a, co
     if (a.slots == 0) S = fwd_split<D>(p, sms, dev);
   }
   const int fit = S > 1 ? fwd_max_clusters<D>(dev, S) : sms;
-  const int workers = static_cast<int>(items < fit ? items : fit);
+  const int workers = p.n_items < fit ? p.n_items : fit;
   p.plane_block =
       model::causal_block_layout(planes, (a.Hq / a.Hkv) >> lg, a.Skv, D, p.n_pairs, workers, &p.last_h0);
   if constexpr (PACKED) {
@@ -2261,7 +2289,7 @@ cudaError_t launch_design(Kernel kernel, int rows_per_item, const FwdArgs& a, co
     }
   }
   // (a causal launch of one round has no order of CTAs to keep: see launch_dependent)
-  return launch_dependent(!a.causal || items <= sms, kernel, workers, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
+  return launch_dependent(!a.causal || p.n_items <= sms, kernel, workers, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
 }
 
 // Ring depths compiled for the block-size ablation of the two-tile design (the model's
@@ -2325,6 +2353,12 @@ cudaError_t launch_fwd_d(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t st
 cudaError_t launch_fwd(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t stream) {
   if (a.D == 128) return launch_fwd_d<128>(a, ctl, stream);
   return launch_fwd_d<64>(a, ctl, stream);
+}
+
+int fwd_cluster_of(const FwdArgs& a) {
+  const int model_design = a.D == 128 ? model::fwd_plan(128).design : model::fwd_plan(64).design;
+  if ((a.design ? a.design : model_design) != 2 || a.slots != 0) return 1;
+  return a.D == 128 ? fwd_cluster<128>(a) : fwd_cluster<64>(a);
 }
 
 cudaError_t launch_fwd_varlen(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaStream_t stream) {

@@ -136,5 +136,7 @@ int decode_max_clusters(int D, int G, int cs);
 // cache, D = 128, 4 query heads per kv head), 0 if that plan is not compiled.
 int decode_ablation_plan(int tokens, int stages, int ctas_per_sm);
 cudaError_t launch_fwd(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t stream);
+// CTAs per cluster that share a work item of launch_fwd (1: no cluster, 0: unknown).
+int fwd_cluster_of(const FwdArgs& a);
 
 }  // namespace loom

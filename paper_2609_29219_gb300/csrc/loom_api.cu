@@ -122,6 +122,16 @@ loom_status loom_attn_fwd(const void* q, const void* k, const void* v, void* o, 
                                                                                : LOOM_ERR_CUDA;
 }
 
+int loom_attn_fwd_cluster(int B, int Hq, int Hkv, int Sq, int Skv, int D, int causal) {
+  if (B <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv || Sq <= 0 || Skv <= 0 || (D != 64 && D != 128)) return 0;
+  if ((causal != 0 && causal != 1) || (causal && Sq > Skv) || static_cast<long long>(B) * Hq > 0x7fffffff) return 0;
+  const FwdArgs a{nullptr, nullptr, nullptr, nullptr, nullptr, B, Hq, Hkv, Sq, Skv, D, causal, 1.f, g_prefill_design,
+                  g_prefill_slots};
+  const int n = fwd_cluster_of(a);
+  cudaGetLastError();
+  return n;
+}
+
 int loom_attn_decode_num_splits(int B, int Hq, int Hkv, int Skv, int D) {
   if (B <= 0 || Hq <= 0 || Hkv <= 0 || Skv <= 0 || Hq % Hkv != 0) return 0;
   if (D != 64 && D != 128) return 0;

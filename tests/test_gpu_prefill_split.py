@@ -52,6 +52,41 @@ def test_few_items(loom, B, Hq, Hkv, Sq, Skv, D, causal):
     assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy(), lse_ref, f"{(B, Hq, Hkv, Sq, Skv, D, causal)}")
 
 
+# Clusters that take several items in turn (more items than the SMs hold clusters at once)
+# of 2 and 4: the last item of a plane has one tile; causal items so short that a CTA of the
+# cluster has no keys of them; both; neither
+ROUNDS = [
+    (1, 12, 1, 1673, 1799, 64, True, 2), (1, 12, 1, 1779, 1827, 128, True, 2), (1, 8, 1, 2503, 2595, 64, True, 2),
+    (1, 16, 2, 1636, 1698, 128, True, 2), (3, 32, 32, 259, 5340, 64, False, 2), (1, 4, 4, 3392, 5663, 64, True, 4),
+    (1, 4, 4, 3253, 3715, 128, True, 4),
+]
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,causal,cluster", ROUNDS)
+def test_several_items_per_cluster(loom, B, Hq, Hkv, Sq, Skv, D, causal, cluster):
+    import torch
+    assert loom.loom_attn_fwd_cluster(B, Hq, Hkv, Sq, Skv, D, causal) == cluster
+    group = Hq // Hkv
+    packed = group & -group  # heads whose rows share query tiles: the group's power of two
+    items = B * Hq // packed * -(-Sq * packed // 256)
+    assert items * cluster > torch.cuda.get_device_properties(0).multi_processor_count
+    q = synth.bf16_normal(7, synth.STREAM_Q, (B, Hq, Sq, D))
+    k = synth.bf16_normal(7, synth.STREAM_K, (B, Hkv, Skv, D))
+    v = synth.bf16_normal(7, synth.STREAM_V, (B, Hkv, Skv, D))
+    qd, kd, vd = to_dev(q), to_dev(k), to_dev(v)
+    first = None
+    for _ in range(30):  # the same bits each time: nothing depends on the order the CTAs run in
+        o = torch.full((B, Hq, Sq, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((B, Hq, Sq), float("nan"), device="cuda")
+        loom.loom_attn_fwd(qd, kd, vd, o, lse, causal=causal)
+        if first is None:
+            first = o, lse
+        assert torch.equal(o.view(torch.int16), first[0].view(torch.int16)) and torch.equal(lse, first[1])
+    loom.loom_attn_check_error()
+    o_ref, lse_ref = oracle.attention(q, k, v, causal=causal)
+    assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy(), lse_ref, f"{(B, Hq, Hkv, Sq, Skv, D, causal)}")
+
+
 def test_extreme_scores_across_shares(loom):
     """Rows whose largest scores lie in one CTA's share: the other shares' weights underflow
     to zero (their partials must not bring in NaN or infinity)."""
