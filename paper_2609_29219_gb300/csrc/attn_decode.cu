@@ -2182,15 +2182,16 @@ cudaError_t launch_ablation(const DecodeArgs& a, const KernelCtl& ctl, cudaStrea
 template <int D, int GT, bool PAGED>
 cudaError_t launch_form(const DecodeArgs& args, const PagedKV* pk, const KernelCtl& ctl, cudaStream_t stream) {
   DecodeArgs a = args;
-  if (D == 128 && GT == 4 && !PAGED && a.stage_plan > 0) return launch_ablation(a, ctl, stream);
+  const bool ablation = D == 128 && GT == 4 && !PAGED && a.stage_plan > 0;
   int cs = 0;
-  const int form = decode_form<D, GT, PAGED>(a, &cs);
-  const bool tc_persist =
-      form == kDecodeSplitMerge && decode_tc_eligible(a) && a.tc != 2;  // counts splits by the lengths
+  const int form = ablation ? kDecodeSplitMerge : decode_form<D, GT, PAGED>(a, &cs);
+  // only the tensor cores' persistent split kernel counts splits by the lengths
+  const bool tc_persist = !ablation && form == kDecodeSplitMerge && decode_tc_eligible(a) && a.tc != 2;
   if (!tc_persist && a.equal_splits > 0) {
     a.splits = a.equal_splits;
     a.equal_splits = 0;
   }
+  if (ablation) return launch_ablation(a, ctl, stream);
   if (form == kDecodeCluster) return launch_cluster<D, GT, PAGED>(a, cs, pk, ctl, stream);
   cudaError_t e;
   if (form == kDecodePersistent)

@@ -81,3 +81,35 @@ def test_smaller_workspace_keeps_the_models_count(loom):
     o_ref, lse_ref = oracle.attention(q, k, v, seqlens_k=lens)
     assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy().reshape(lse_ref.shape), lse_ref, "small workspace")
     assert bool((ws[need:] == 0x7F).all())
+
+
+@pytest.mark.parametrize("what", ["plan 32x2x2", "plan 128x3x1", "CUDA cores", "one CTA per split", "persistent", "cluster"])
+def test_other_kernels_keep_the_models_count(loom, what):
+    """Kernels that do not count splits by the lengths take the model's, on the same workspace."""
+    import torch
+    B, Hq, Hkv, Skv, D = 16, 32, 8, 2048, 128
+    n = loom.loom_attn_decode_num_splits(B, Hq, Hkv, Skv, D)
+    assert (loom.loom_attn_decode_workspace_bytes(B, Hq, Hkv, Skv, D, 0) >
+            loom.loom_attn_decode_workspace_bytes(B, Hq, Hkv, Skv, D, n))  # a batch that has two counts
+    q = synth.bf16_normal(6, synth.STREAM_Q, (B, Hq, 1, D))
+    k = synth.bf16_normal(6, synth.STREAM_K, (B, Hkv, Skv, D))
+    v = synth.bf16_normal(6, synth.STREAM_V, (B, Hkv, Skv, D))
+    lens = _lens("ramp", B, Skv)
+    o_ref, lse_ref = oracle.attention(q, k, v, seqlens_k=lens)
+    qd, kd, vd, ld = to_dev(q), to_dev(k), to_dev(v), torch.from_numpy(lens).cuda()
+    try:
+        if what.startswith("plan"):
+            assert loom.loom_debug_decode_stage_plan(*map(int, what.split()[1].split("x")))
+        elif what in ("persistent", "cluster"):
+            loom.loom_debug_decode_form(2 if what == "persistent" else 3)
+        else:
+            loom.loom_debug_decode_tensor_cores(0 if what == "CUDA cores" else 2)
+        need = loom.loom_attn_decode_workspace_bytes(B, Hq, Hkv, Skv, D, 0)
+        ws = torch.zeros(need, dtype=torch.uint8, device="cuda")
+        o, lse = loom.loom_attn_decode(qd, kd, vd, ld, workspace=ws, return_lse=True)
+        loom.loom_attn_check_error()
+    finally:
+        loom.loom_debug_decode_stage_plan(0)
+        loom.loom_debug_decode_form(0)
+        loom.loom_debug_decode_tensor_cores(1)
+    assert_parity(o_to_f64(o), o_ref, lse.cpu().numpy().reshape(lse_ref.shape), lse_ref, what)
