@@ -61,12 +61,11 @@ struct GemmCfg {
 };
 
 // The split-K kernel for at most 32 rows of C: a stage's A tile is 4 KB (the MMA's other 96
-// rows read on into the stage's B tile and past it, in this CTA's shared memory, and only
-// reach accumulator rows that C does not have), and the ring is half an SM's shared memory,
-// so that two CTAs share an SM: the next launch's CTAs, or the other half of the splits, are
-// there when this one's first bytes are still on their way.  It needs two CTAs on many of the
-// SMs to keep as many bytes in flight as one of the large ring does (kSkinnyMinCtas).
-constexpr int kSkinnyRows = 32, kSkinnyMinCtas = 176;
+// rows read on into the stage's B tile and only reach accumulator rows that C does not
+// have), and the ring is half an SM's shared memory, so that two CTAs share an SM: the next
+// launch's CTAs, or the other half of the splits, are there when this one's first bytes are
+// still on their way (see skinny_fits).
+constexpr int kSkinnyRows = 32;
 template <int BN>
 struct GemmSkinnyCfg {
   static constexpr int BM = 128, BK = 64, A_ROWS = kSkinnyRows;
@@ -75,15 +74,15 @@ struct GemmSkinnyCfg {
   static constexpr uint32_t A_BYTES = A_ROWS * BK * 2;
   static constexpr uint32_t B_BOX_BYTES = BK * 64 * 2;
   static constexpr uint32_t STAGE_BYTES = A_BYTES + NB * B_BOX_BYTES;
-  static constexpr uint32_t PAST_BYTES = STAGE_BYTES < BM * BK * 2 ? BM * BK * 2 - STAGE_BYTES : 0;
-  static constexpr int NSTAGE = (112 * 1024 - static_cast<int>(PAST_BYTES)) / static_cast<int>(STAGE_BYTES + 512);
+  static constexpr int NSTAGE = 112 * 1024 / static_cast<int>(STAGE_BYTES + 512);
   static constexpr uint32_t STG_OFF = NSTAGE * STAGE_BYTES;
-  static constexpr uint32_t BAR_OFF = STG_OFF + PAST_BYTES;
+  static constexpr uint32_t BAR_OFF = STG_OFF;
   static constexpr int NBAR = 2 * NSTAGE + 5;
   static constexpr uint32_t TMEM_PTR_OFF = BAR_OFF + NBAR * 8;
   static constexpr uint32_t ABORT_OFF = TMEM_PTR_OFF + 8;
   static constexpr uint32_t BYTES = ABORT_OFF + 16 + 1024;  // + alignment slack
   static_assert(STAGE_BYTES % 1024 == 0, "swizzled tiles start on the swizzle period");
+  static_assert(STAGE_BYTES >= BM * BK * 2, "the MMA's 128 rows of A stay in the stage");
   static_assert(2 * (BYTES + 1024) <= 228 * 1024, "two CTAs per SM");
 };
 
@@ -957,7 +956,7 @@ bool prepare_splitk(int dev) {
 
 // CTAs of clusters of S that fit on the device at once (0: none, or cannot be queried); both
 // B layouts have the same resources, so the [K, N] instance answers for both.
-template <int BN>
+template <int BN, class C = GemmCfg<BN>>
 int splitk_slots(int dev, int S) {
   static std::atomic<int> cache[kSlotCacheDevices][5];  // [device][log2 S], value + 1 once known
   int lg = 0;
@@ -969,10 +968,10 @@ int splitk_slots(int dev, int S) {
     if (c != 0) return c - 1;
   }
   int clusters = 0;
-  if (prepare_splitk<BN, false>(dev)) {
+  if (prepare_splitk<BN, false, C>(dev)) {
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = splitk_config<BN>(S * 64, S, nullptr, attr);
-    if (cudaOccupancyMaxActiveClusters(&clusters, gemm_splitk_kernel<BN, false>, &cfg) != cudaSuccess) {
+    cudaLaunchConfig_t cfg = splitk_config<BN, C>(S * 64, S, nullptr, attr);
+    if (cudaOccupancyMaxActiveClusters(&clusters, gemm_splitk_kernel<BN, false, C>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       clusters = 0;
     }
@@ -990,6 +989,35 @@ int splitk_slots_any(int dev, int bn, int S) {
   }
 }
 
+// Whether S splits over 128-wide tiles run on the kernel for at most 32 rows (GemmSkinnyCfg):
+//   - it needs two CTAs on many of the SMs to keep as many bytes in flight as one of the large
+//     ring does: 23 CTAs for every 20 SMs or more;
+//   - all clusters must be resident at once, two CTAs per SM (the query counts one): with one
+//     more the launch takes two rounds.  B [N, K], N 8960 (70 tiles) K 8448 at S = 4 25.9 us
+//     against 26.7 on the model's choice, but N 9616 (76; 72 fit) 43.8 against 33.2; at S = 16
+//     N 1680 (14) 13.8 / 15.3, N 2048 (16; 14 fit) 22.3 / 17.4;
+//   - rows of A and B that start on a 32-byte sector (K and N multiples of 16, whichever way B
+//     lies): where they do not, the copies wait longer and the large ring hides more of it (M 16
+//     N 6184 K 10408 26.4 / 23.2, M 17 N 12344 K 7632 35.7 / 32.4).
+// GB300, weights read from HBM, this against the model's choice over 64 shapes whose clusters
+// fit and whose rows of B start on a sector: B [N, K] 1.01 to 1.14 times as fast (geomean 1.07),
+// B [K, N] 0.96 to 1.11 (1.05).  With a weight that a program finds in L2 again, the model's
+// 192-wide tiles are as much faster (M 16 N 6144 K 4096 8.5 / 8.0); weights are read from HBM.
+template <int BN>
+bool skinny_fits(int M, int N, int K, int S, int dev, int sms) {
+  const long long ctas = static_cast<long long>((N + BN - 1) / BN) * S;
+  if (M > kSkinnyRows || N % 16 != 0 || K % 16 != 0 || 20 * ctas < 23ll * sms || ctas > 2ll * sms) return false;
+  return ctas <= 2ll * splitk_slots<BN, GemmSkinnyCfg<BN>>(dev, S);
+}
+
+// The most splits of 16 K stages or more each that it takes; 0: none, the model chooses.
+// (M 16 N 6144 K 4096: 13.1 us on the model's choice, 12.4 on this.)
+int skinny_splits(int M, int N, int K, int dev, int sms) {
+  for (int S = 16; S >= 2; S /= 2)
+    if ((K + 63) / 64 >= 16 * S && skinny_fits<128>(M, N, K, S, dev, sms)) return S;
+  return 0;
+}
+
 template <int BN, bool BKM, class C>
 cudaError_t launch_splitk_cfg(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stream, int dev, int S) {
   if (!prepare_splitk<BN, BKM, C>(dev)) return cudaErrorInvalidValue;
@@ -1005,9 +1033,9 @@ cudaError_t launch_splitk_cfg(const GemmArgs& a, const KernelCtl& ctl, cudaStrea
 }
 
 template <int BN, bool BKM>
-cudaError_t launch_splitk(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stream, int dev, int S) {
+cudaError_t launch_splitk(const GemmArgs& a, const KernelCtl& ctl, cudaStream_t stream, int dev, int sms, int S) {
   if constexpr (BN == 128) {
-    if (a.M <= kSkinnyRows && static_cast<long long>((a.N + BN - 1) / BN) * S >= kSkinnyMinCtas)
+    if (skinny_fits<BN>(a.M, a.N, a.K, S, dev, sms))
       return launch_splitk_cfg<BN, BKM, GemmSkinnyCfg<BN>>(a, ctl, stream, dev, S);
   }
   return launch_splitk_cfg<BN, BKM, GemmCfg<BN>>(a, ctl, stream, dev, S);
@@ -1130,10 +1158,10 @@ cudaError_t launch_choice(const GemmArgs& a, const GemmChoice& c, const KernelCt
   if (c.pair == 1) return launch_pair<BKM>(a, ctl, stream, dev);
   if (c.splits > 1) {
     switch (c.tile_n) {
-      case 64: return launch_splitk<64, BKM>(a, ctl, stream, dev, c.splits);
-      case 128: return launch_splitk<128, BKM>(a, ctl, stream, dev, c.splits);
-      case 192: return launch_splitk<192, BKM>(a, ctl, stream, dev, c.splits);
-      default: return launch_splitk<256, BKM>(a, ctl, stream, dev, c.splits);
+      case 64: return launch_splitk<64, BKM>(a, ctl, stream, dev, sms, c.splits);
+      case 128: return launch_splitk<128, BKM>(a, ctl, stream, dev, sms, c.splits);
+      case 192: return launch_splitk<192, BKM>(a, ctl, stream, dev, sms, c.splits);
+      default: return launch_splitk<256, BKM>(a, ctl, stream, dev, sms, c.splits);
     }
   }
   switch (c.tile_n) {
@@ -1142,19 +1170,6 @@ cudaError_t launch_choice(const GemmArgs& a, const GemmChoice& c, const KernelCt
     case 192: return launch_bn<192, BKM>(a, ctl, stream, dev, sms);
     default: return launch_bn<256, BKM>(a, ctl, stream, dev, sms);
   }
-}
-
-// Splits of the split-K kernel for at most 32 rows over 128-wide tiles: the most that two CTAs
-// per SM hold, of 16 K stages or more each; 0 where that leaves fewer than kSkinnyMinCtas,
-// and the model's choice with the large ring is as fast.  GB300, weights read from HBM, us,
-// the model's choice / this: M 16 N 6144 K 4096 13.1 / 12.4, M 16 N 16384 K 4096 27.3 / 26.1,
-// M 32 N 12288 K 4096 22.3 / 20.7, M 3 N 5600 K 11432 26.5 / 25.5; not taken: M 1 N 4096 K 4096
-// 9.0 / 9.2, M 8 9.0 / 9.9.
-int skinny_splits(int N, int K, int sms) {
-  const long long tiles = (N + 127) / 128, stages = (K + 63) / 64;
-  for (int S = 16; S >= 2; S /= 2)
-    if (tiles * S <= 2ll * sms && stages >= 16ll * S) return tiles * S >= kSkinnyMinCtas ? S : 0;
-  return 0;
 }
 
 bool device_sms(int* dev, int* sms) {
@@ -1167,8 +1182,8 @@ bool device_sms(int* dev, int* sms) {
 GemmChoice gemm_choice(int M, int N, int K, GemmChoice forced) {
   int dev = 0, sms = 0;
   if (!device_sms(&dev, &sms)) return {0, 0};
-  if (forced.tile_n == 0 && forced.splits == 0 && forced.pair == 0 && M <= kSkinnyRows) {
-    const int S = skinny_splits(N, K, sms);
+  if (forced.tile_n == 0 && forced.splits == 0 && forced.pair == 0) {
+    const int S = skinny_splits(M, N, K, dev, sms);
     if (S > 0) return {128, S, 0};
   }
   const model::GemmChoiceModel c = model::gemm_choose(

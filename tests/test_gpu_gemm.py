@@ -150,6 +150,31 @@ def test_skinny(loom, M, N, K):
     _check(c.float().cpu().numpy().astype(np.float64), c_ref, K, f"skinny M={M} N={N} K={K} transposed")
 
 
+@pytest.mark.parametrize("M", [1, 17, 32])
+@pytest.mark.parametrize("N,K,splits", [(6144, 4096, 4), (11264, 2064, 2), (3584, 8208, 8), (1536, 16400, 16)])
+def test_skinny_split_counts(loom, M, N, K, splits):
+    """Every split count of the kernel with the small ring, in both layouts of B."""
+    import torch
+    assert (loom.loom_gemm_tile_n(M, N, K), loom.loom_gemm_splits(M, N, K)) == (128, splits)
+    a, b = _inputs(M + N, M, K, N)
+    c_ref = oracle.gemm(a, b)
+    bd = to_dev(b)
+    for bt in (False, True):
+        guard = torch.full((M + 8, N), 7.0, dtype=torch.bfloat16, device="cuda")
+        c = loom.loom_gemm_bf16(to_dev(a), bd.t().contiguous() if bt else bd, guard[:M], b_transposed=bt)
+        loom.loom_attn_check_error()
+        _check(c.float().cpu().numpy().astype(np.float64), c_ref, K, f"M={M} N={N} K={K} S={splits} bt={bt}")
+        assert bool((guard[M:] == 7.0).all())
+
+
+@pytest.mark.parametrize("N,K", [(9600, 4480), (4096, 8192), (2048, 16384), (6152, 4096), (6144, 4104)])
+def test_skinny_refused(loom, N, K):
+    """More clusters than fit at once, or rows off the 32-byte sector: 16 rows are split as 33
+    are or by fewer, on another tile width or count than the small ring's."""
+    s = next(s for s in (16, 8, 4, 2) if -(-N // 128) * s <= 304 and -(-K // 64) >= 16 * s)
+    assert (loom.loom_gemm_tile_n(16, N, K), loom.loom_gemm_splits(16, N, K)) != (128, s)
+
+
 @pytest.mark.parametrize("splits", SPLITS, ids=[f"s{s}" for s in SPLITS])
 def test_split_with_idle_ctas(loom, forced, splits):
     """K = 64 is one stage: all but one CTA of each cluster get no stage and add zeros."""
