@@ -183,7 +183,8 @@ def _torch():
         import torch
         try:  # what torch's generated code allocates by: no dispatch, on the current device
             from torch._C._dynamo.guards import _empty_strided_cuda as call
-            if hasattr(torch._C, "_cuda_getDevice"):
+            if all(hasattr(torch._C, n) for n in ("_cuda_getDevice", "_len_torch_dispatch_stack",
+                                                  "_len_torch_function_stack", "_get_deterministic_algorithms")):
                 _empty_strided_cuda = call
         except ImportError:
             pass
@@ -191,12 +192,18 @@ def _torch():
     return _torch_mod
 
 
-def _new(shape, strides, dtype, t):
-    """An uninitialised contiguous tensor (strides: its strides) on CUDA tensor t's device."""
+def _new(shape, strides, dtype, t, like=False):
+    """An uninitialised contiguous tensor (strides: its strides) on CUDA tensor t's device
+    (like: of t's shape and type).  It passes torch's dispatcher by only where nobody would
+    miss the call: no dispatch or function mode, no deterministic mode (which fills new
+    tensors), no subclass of Tensor."""
     torch = _torch_mod
-    if _empty_strided_cuda is not None and t.get_device() == torch._C._cuda_getDevice():
+    c = torch._C
+    if (_empty_strided_cuda is not None and type(t) is torch.Tensor and not c._len_torch_dispatch_stack()
+            and not c._len_torch_function_stack() and not c._get_deterministic_algorithms()
+            and t.get_device() == c._cuda_getDevice()):
         return _empty_strided_cuda(shape, strides, dtype)
-    return torch.empty(shape, dtype=dtype, device=t.device)
+    return torch.empty_like(t) if like else torch.empty(shape, dtype=dtype, device=t.device)
 
 
 def _ptr(t, name, dtype, ndim):
@@ -261,7 +268,7 @@ def loom_attn_fwd(q, k, v, o=None, lse=None, *, causal=False, scale=None, stream
     if v.shape != k.shape or Bk != B or Dk != D:
         raise ValueError("q/k/v shapes disagree")
     if o is None:
-        o = _new((B, Hq, Sq, D), (Hq * Sq * D, Sq * D, D, 1), bf16, q)
+        o = _new((B, Hq, Sq, D), (Hq * Sq * D, Sq * D, D, 1), bf16, q, True)
     if o.shape != q.shape:
         raise ValueError("o must have q's shape")
     op = _ptr(o, "o", bf16, 4)
@@ -305,7 +312,7 @@ def _decode_operands(q, k_cache, v_cache, seqlens_k, o, lse, return_lse):
             raise ValueError("seqlens_k must be [B]")
         sp = _ptr(seqlens_k, "seqlens_k", torch.int32, 1)
     if o is None:
-        o = _new((B, Hq, 1, D), (Hq * D, D, D, 1), bf16, q)
+        o = _new((B, Hq, 1, D), (Hq * D, D, D, 1), bf16, q, True)
     op = _ptr(o, "o", bf16, 4)
     if lse is None and return_lse:
         lse = _new((B, Hq), (Hq, 1), torch.float32, q)
@@ -374,7 +381,7 @@ def loom_attn_fwd_varlen(q, k, v, cu_seqlens_q, cu_seqlens_k, max_seqlen_q, o=No
         raise ValueError("cu_seqlens_q and cu_seqlens_k must both be [B + 1]")
     B = cu_seqlens_q.numel() - 1
     if o is None:
-        o = _new((total_q, Hq, D), (Hq * D, D, 1), bf16, q)
+        o = _new((total_q, Hq, D), (Hq * D, D, 1), bf16, q, True)
     op = _ptr(o, "o", bf16, 3)
     if lse is None and return_lse:
         lse = _new((Hq, total_q), (total_q, 1), torch.float32, q)
@@ -420,7 +427,7 @@ def loom_attn_decode_paged(q, k_cache, v_cache, block_table, seqlens_k, o=None, 
         raise ValueError("seqlens_k must be [B]")
     sp = _ptr(seqlens_k, "seqlens_k", torch.int32, 1)
     if o is None:
-        o = _new((B, Hq, 1, D), (Hq * D, D, D, 1), bf16, q)
+        o = _new((B, Hq, 1, D), (Hq * D, D, D, 1), bf16, q, True)
     op = _ptr(o, "o", bf16, 4)
     if lse is None and return_lse:
         lse = _new((B, Hq), (Hq, 1), torch.float32, q)
