@@ -902,34 +902,44 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
 // the lengths differ (which only the device knows) few items per CTA are as uneven as the
 // lengths: B16 of 4096 to 8192 keys at the model's 2 splits is 256 items on 304 CTAs, the
 // longest twice the shortest.  So the launch carries two counts, that one (`equal`) and a
-// larger one that the partials' space is laid out for (`splits`), and the kernels take the
-// larger one unless the mean length is within 4 % of the longest.  GB300, us, equal / larger
-// count, on unequal lengths and on equal ones (where more items only cost):
-//   B16 Hkv8 4096-8192         2 / 12: 75.0 / 68.1, paged by 16 keys 79.0 / 71.0
-//   B16 Hkv8 8192              2 / 12: 83.1 / 83.9 (2 splits either way: what choosing costs)
-// and not taken (see decode_ragged_splits):
-//   B64 Hkv8 512-2048          1 / 3: 71.1 / 68.3, equal lengths 91.9 / 92.7
-//   B4 Hkv8 4096-8192         8 / 16: 24.2 / 23.1, equal lengths 28.6 / 29.2
-// The split kernel's CTA 0 leaves its count behind the item counter for the merge kernel.
-// Splits of fewer than 65536 / D keys only cost (B48, 100 to 1000 keys: 2 -> 3 splits 31.2 ->
-// 32.4 us).
-
-// By the loader warp, from the B lengths in shared memory.
-__device__ __forceinline__ int ragged_splits(const int* lens, int B, int Skv, int D, int equal, int splits, int lane) {
-  float total = 0.f;
-  int longest = 0;
+// larger one that the partials' space is laid out for (`splits`), and the kernels choose.
+// The split kernel's CTA 0 leaves the choice behind the item counter for the merge kernel.
+//
+// By the loader warp, from the B lengths in shared memory, in stages of 64 keys.  `equal`
+// lasts as long as its longest item.  The larger count lasts as long as its longest item, or,
+// with more items than CTAs, an even share of all keys and one of the shortest items (the
+// last ones dealt), with half a stage (of D = 128) per further round and three for choosing
+// and the merge.  It is taken where that is 15 % less, and never for lengths whose mean is
+// within 4 % of the longest.  GB300, both counts timed on 376 batches that have them, evenly
+// spaced lengths from 90, 50 and 6 % of the longest up: the larger one always is 1.133 times
+// as fast (geomean), but down to 0.76 where a few items make a second round and 0.94 with short
+// sequences (B12 Hkv16 736 to 1472 keys, 1 / 2 splits: 31.9 / 34.1 us); by this rule 1.140, one
+// batch below 0.985 (0.976), and 1.145 with the better of both.  B16 Hkv8 4096 to 8192 keys, 2 /
+// 12 splits: 75.7 / 68.5 us, paged by 16 keys 79.0 / 71.0.
+template <int D>
+__device__ __forceinline__ int ragged_splits(const int* lens, int B, int Hkv, int Skv, int equal, int splits,
+                                             int ctas, int lane) {
+  unsigned total = 0, longest = 0, shortest = 0xffffffffu;
   for (int b = lane; b < B; b += 32) {
-    const int n = max(0, min(lens[b], Skv));
-    total += static_cast<float>(n);
+    const unsigned n = (static_cast<unsigned>(max(0, min(lens[b], Skv))) + 63u) / 64u;
+    total += n;
     longest = max(longest, n);
+    shortest = min(shortest, n);
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    total += __shfl_xor_sync(0xffffffffu, total, off);
-    longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, off));
+  total = __reduce_add_sync(0xffffffffu, total);
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  shortest = __reduce_min_sync(0xffffffffu, shortest);
+  if (static_cast<float>(total) >= 0.96f * static_cast<float>(longest) * static_cast<float>(B)) return equal;
+  const unsigned n = equal, r = min(splits, static_cast<int>(longest * (D / 64) / 16));  // 65536 / D keys or more
+  if (r <= n) return equal;
+  constexpr float kStage = 128.f / D;
+  float t = static_cast<float>((longest + r - 1) / r);
+  const float rounds = static_cast<float>(B * Hkv * static_cast<int>(r)) / static_cast<float>(ctas);
+  if (rounds > 1.f) {
+    const float even = static_cast<float>(total) * static_cast<float>(Hkv) / static_cast<float>(ctas);
+    t = fmaxf(t, even + static_cast<float>((shortest + r - 1) / r)) + 0.5f * (rounds - 1.f) * kStage;
   }
-  if (total >= 0.96f * static_cast<float>(longest) * static_cast<float>(B)) return equal;
-  return max(equal, min(splits, longest / (65536 / D)));
+  return t + 3.f * kStage < 0.85f * static_cast<float>((longest + n - 1) / n) ? static_cast<int>(r) : equal;
 }
 
 template <int D>
@@ -1147,7 +1157,7 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
     }
     // (by the loader warp, while warp 0 sorts; equal > 0 implies sorted)
     if (warp == 1 && equal > 0) {
-      count = ragged_splits(lens, B, Skv, D, equal, splits, lane);
+      count = ragged_splits<D>(lens, B, Hkv, Skv, equal, splits, static_cast<int>(gridDim.x), lane);
       if (blockIdx.x == 0 && lane == 0) sched[1] = static_cast<unsigned long long>(count);
     }
     __syncthreads();

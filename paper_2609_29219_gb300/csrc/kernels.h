@@ -58,20 +58,24 @@ struct DecodeArgs {
 };
 
 // Split count that the workspace of a call with the model's count `equal` is laid out for: up
-// to five items for each of the 304 CTAs, so that unequal lengths even out, of 65536 / D keys
-// or more.  Only where a sequence has few items and they fill one round: with more of either
-// the dealing evens the lengths out already, and unequal lengths gain no more than the second
-// count costs equal ones (see ragged_splits in attn_decode.cu for the measurements).
+// to five items for each of the split kernel's two CTAs per SM, so that unequal lengths even
+// out, of 65536 / D keys or more (B48, 100 to 1000 keys, 2 / 3 splits: 31.2 / 32.4 us).  Only
+// where a sequence has few items and they fill one round: with more of either the dealing
+// evens the lengths out already (GB300, us, model's count / larger one: B64 Hkv8 512 to 2048
+// keys 1 / 3 splits 71.1 / 68.3, equal lengths 91.9 / 92.7; B4 Hkv8 4096 to 8192 8 / 16: 24.2 /
+// 23.1, equal lengths 28.6 / 29.2).  And only where it is twice the model's: choosing costs 0.2
+// to 0.8 us whichever count is taken, and a smaller difference gains less than that (B54 Hkv2,
+// 777 to 1554 keys, 2 / 3: 23.8 / 24.8; B18 Hkv8, 780 to 1560, 2 / 3: 23.3 / 23.9).
 constexpr int kMaxRaggedB = 256;  // sequences
-inline int decode_ragged_splits(int B, int Hq, int Hkv, int Skv, int D, int equal) {
+inline int decode_ragged_splits(int B, int Hq, int Hkv, int Skv, int D, int equal, int sms) {
   if (B < 2 || B > kMaxRaggedB || Hq / Hkv > 32) return equal;
-  const long long units = static_cast<long long>(B) * Hkv;
-  if (units * equal > 304 || equal > 4) return equal;
-  long long r = (1536 + units - 1) / units;
+  const long long units = static_cast<long long>(B) * Hkv, ctas = 2ll * sms;
+  if (units * equal > ctas || equal > 4) return equal;
+  long long r = (5 * ctas + units - 1) / units;
   const long long most = static_cast<long long>(Skv) * D / 65536;
   if (r > most) r = most;
   if (r > 64) r = 64;  // the merge holds them in registers
-  return r > equal ? static_cast<int>(r) : equal;
+  return r >= 2ll * equal ? static_cast<int>(r) : equal;
 }
 
 // High word of an armed item counter: a signalling-NaN pattern that no float the decode

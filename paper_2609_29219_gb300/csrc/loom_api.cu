@@ -64,6 +64,12 @@ int current_sm_count() {
   return sms;
 }
 
+// The current device's SMs, or the model's count without a device.
+int sms_or_model() {
+  const int sms = current_sm_count();
+  return sms > 0 ? sms : model::kGb300.num_sms;
+}
+
 struct SplitKey {
   int B, Hq, Hkv, Skv, D, sms, tc;
   bool operator==(const SplitKey& o) const {
@@ -135,8 +141,7 @@ int loom_attn_fwd_cluster(int B, int Hq, int Hkv, int Sq, int Skv, int D, int ca
 int loom_attn_decode_num_splits(int B, int Hq, int Hkv, int Skv, int D) {
   if (B <= 0 || Hq <= 0 || Hkv <= 0 || Skv <= 0 || Hq % Hkv != 0) return 0;
   if (D != 64 && D != 128) return 0;
-  int sms = current_sm_count();
-  if (sms <= 0) sms = model::kGb300.num_sms;
+  const int sms = sms_or_model();
   // The enumeration costs ~0.1 ms of host time: remember the answer per problem shape.
   // the split + merge form's split kernel runs on the tensor cores for a contiguous cache
   // (a paged cache takes the same split count, with the CUDA-core kernel)
@@ -170,7 +175,7 @@ int loom_attn_decode_num_splits(int B, int Hq, int Hkv, int Skv, int D) {
 size_t loom_attn_decode_workspace_bytes(int B, int Hq, int Hkv, int Skv, int D, int num_splits) {
   if (num_splits == 0) {
     num_splits = loom_attn_decode_num_splits(B, Hq, Hkv, Skv, D);
-    if (num_splits > 0) num_splits = decode_ragged_splits(B, Hq, Hkv, Skv, D, num_splits);
+    if (num_splits > 0) num_splits = decode_ragged_splits(B, Hq, Hkv, Skv, D, num_splits, sms_or_model());
   }
   if (num_splits <= 0 || num_splits > kMaxDecodeSplits) return 0;
   if (B <= 0 || Hq <= 0 || (D != 64 && D != 128)) return 0;
@@ -212,7 +217,7 @@ namespace {
 // model's is returned (0: nothing changes).
 int ragged_layout(bool lengths, int B, int Hq, int Hkv, int Skv, int D, size_t workspace_bytes, int* splits) {
   if (!lengths) return 0;
-  const int r = decode_ragged_splits(B, Hq, Hkv, Skv, D, *splits);
+  const int r = decode_ragged_splits(B, Hq, Hkv, Skv, D, *splits, sms_or_model());
   if (r == *splits || decode_workspace_bytes(B, Hq, D, r) > workspace_bytes) return 0;
   const int equal = *splits;
   *splits = r;

@@ -63,6 +63,27 @@ def test_ragged_splits(loom, kind, B, Hq, Hkv, Skv, D, splits):
     assert bool((ws[need:] == 0x7F).all())
 
 
+@pytest.mark.parametrize("B,Hkv,Skv,lo,larger", [
+    (16, 8, 8192, 1.0, False), (16, 8, 8192, 0.98, False),  # one length, nearly
+    (16, 8, 8192, 0.5, True), (11, 16, 5211, 0.9, True),    # uneven; too few items of one length each
+    (28, 8, 2567, 0.9, False), (16, 8, 2048, 0.5, False),   # a last round with few items in it
+    (16, 8, 8192, 0.0, True)])
+def test_count_taken(loom, B, Hkv, Skv, lo, larger):
+    """The count that the split kernel leaves behind the item counter for the merge kernel."""
+    import torch
+    D = 128
+    n = loom.loom_attn_decode_num_splits(B, 2 * Hkv, Hkv, Skv, D)
+    need = loom.loom_attn_decode_workspace_bytes(B, 2 * Hkv, Hkv, Skv, D, 0)
+    ws = torch.zeros(need, dtype=torch.uint8, device="cuda")
+    q = torch.randn((B, 2 * Hkv, 1, D), device="cuda", dtype=torch.bfloat16)
+    kv = torch.randn((B, Hkv, Skv, D), device="cuda", dtype=torch.bfloat16)
+    lens = torch.linspace(lo * Skv, Skv, B).round().int().cuda()
+    loom.loom_attn_decode(q, kv, kv, lens, workspace=ws)
+    loom.loom_attn_check_error()
+    count = int(ws[need - 256:].view(torch.int64)[1])
+    assert (n < count <= 64) if larger else count == n
+
+
 def test_smaller_workspace_keeps_the_models_count(loom):
     """A workspace of the model's own count, as num_splits names it, is still enough."""
     import torch
