@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
 // larger one that the partials' space is laid out for (`splits`), and the kernels choose.
 // The split kernel's CTA 0 leaves the choice behind the item counter for the merge kernel.
 //
-// By the loader warp, from the B lengths in shared memory, in stages of 64 keys.  `equal`
+// By the MMA warp, from the B lengths in shared memory, in stages of 64 keys.  `equal`
 // lasts as long as its longest item.  The larger count lasts as long as its longest item, or,
 // with more items than CTAs, an even share of all keys and one of the shortest items (the
 // last ones dealt), with half a stage (of D = 128) per further round and three for choosing
@@ -930,22 +930,33 @@ __device__ __forceinline__ int ragged_splits(const int* lens, int B, int Hkv, in
   longest = __reduce_max_sync(0xffffffffu, longest);
   shortest = __reduce_min_sync(0xffffffffu, shortest);
   if (static_cast<float>(total) >= 0.96f * static_cast<float>(longest) * static_cast<float>(B)) return equal;
-  const unsigned n = equal, r = min(splits, static_cast<int>(longest * (D / 64) / 16));  // 65536 / D keys or more
-  if (r <= n) return equal;
+  const int r = min(splits, static_cast<int>(longest * (D / 64) / 16));  // 65536 / D keys or more
+  if (r <= equal) return equal;
+  // (quotients of approximate division: every CTA has the same, and a count hangs on them, no result)
   constexpr float kStage = 128.f / D;
-  float t = static_cast<float>((longest + r - 1) / r);
-  const float rounds = static_cast<float>(B * Hkv * static_cast<int>(r)) / static_cast<float>(ctas);
-  if (rounds > 1.f) {
-    const float even = static_cast<float>(total) * static_cast<float>(Hkv) / static_cast<float>(ctas);
-    t = fmaxf(t, even + static_cast<float>((shortest + r - 1) / r)) + 0.5f * (rounds - 1.f) * kStage;
-  }
-  return t + 3.f * kStage < 0.85f * static_cast<float>((longest + n - 1) / n) ? static_cast<int>(r) : equal;
+  const float all = static_cast<float>(longest), part = __fdividef(1.f, static_cast<float>(r));
+  const float per_cta = __fdividef(static_cast<float>(Hkv), static_cast<float>(ctas));
+  const float rounds = static_cast<float>(B * r) * per_cta;
+  auto whole = [](float stages) { return ceilf(stages - 1e-3f); };
+  float t = whole(all * part);
+  if (rounds > 1.f)
+    t = fmaxf(t, static_cast<float>(total) * per_cta + whole(static_cast<float>(shortest) * part)) +
+        0.5f * (rounds - 1.f) * kStage;
+  return t + 3.f * kStage < 0.85f * whole(__fdividef(all, static_cast<float>(equal))) ? r : equal;
 }
 
 template <int D>
 struct DecodeTcPersistCfg {
   using C = DecodeTcCfg<D>;
   static constexpr int kMaxSortedB = kMaxRaggedB;         // sequences sorted by length
+  // Stages that a CTA has still to issue when it lets the merge grid launch, where it has one
+  // item of a batch of several sequences: the CTA of the longest works on alone, and after its
+  // last copy too little time is left to hide the launch.  GB300, us, launched at the start / at
+  // 0 / 10 / 24 stages: lengths from half the longest up, B32 H64/8 2977 keys 63.4 / 64.2 / 63.0 /
+  // 62.8, B18 H64/8 3049 keys 39.4 / 40.0 / 39.3 / 39.5; one length, B32 H64/8 2977 keys 70.1 / 70.5 /
+  // 70.5 / 70.5.  Several items per CTA end together: 0 is better (B16 4096 to 8192 keys of 16 in a
+  // page at 12 splits 71.2, at 10 stages 72.0).
+  static constexpr int kMergeLead = 10;
   static constexpr uint32_t Q_BOX_BYTES = C::MAX_G * 128;  // up to 32 heads x 64 dims
   static constexpr uint32_t Q_OFF = C::NSTAGE * C::STAGE_BYTES;
   static constexpr uint32_t META_OFF = Q_OFF + C::NBOX * Q_BOX_BYTES;  // [NSTAGE] x 8 int32
@@ -956,6 +967,7 @@ struct DecodeTcPersistCfg {
   static constexpr int NBAR = 2 * C::NSTAGE + 7;
   static constexpr uint32_t TMEM_PTR_OFF = BAR_OFF + NBAR * 8;
   static constexpr uint32_t ABORT_OFF = TMEM_PTR_OFF + 8;
+  static constexpr uint32_t COUNT_OFF = ABORT_OFF + 8;  // int32: the splits of every sequence
   static constexpr uint32_t BYTES = ABORT_OFF + 16 + 1024;  // + 1024-byte alignment slack
   static_assert(Q_OFF % 1024 == 0 && Q_BOX_BYTES % 1024 == 0, "q boxes start on the swizzle period");
   static_assert(2 * (BYTES + 1024) <= 228 * 1024 && 3 * (BYTES + 1024) > 228 * 1024, "exactly two CTAs per SM");
@@ -983,7 +995,7 @@ __device__ __forceinline__ void decode_tc_persist_rows(const uint8_t* smem, floa
     const volatile int* rec = reinterpret_cast<const volatile int*>(smem + L::META_OFF + slot * 32);
     const int b = rec[0];
     if (b < 0) return;  // no more items
-    const int hk = rec[1], split = rec[2], j = rec[3], n_st = rec[4], ntok = rec[6], splits = rec[7];
+    const int hk = rec[1], split = rec[2], j = rec[3], n_st = rec[4], ntok = rec[6];
     if (j == 0) {
       if (!mbar_wait_warp(bar_qf, nq & 1, ctl, ab)) return;
 #pragma unroll
@@ -1055,6 +1067,7 @@ __device__ __forceinline__ void decode_tc_persist_rows(const uint8_t* smem, floa
       // the item's last P.V, then O / l and the log-sum-exp of each real row
       if (!mbar_wait_warp(bar_o, st & 1, ctl, ab)) return;
       tc_fence_after();
+      const int splits = reinterpret_cast<const volatile int*>(smem + L::COUNT_OFF)[0];
       const size_t row0 = (static_cast<size_t>(b) * Hq + static_cast<size_t>(hk) * G) * splits + split;
       const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
       float* dst = o_part + (row0 + static_cast<size_t>(real ? lane : 0) * splits) * D;
@@ -1126,6 +1139,7 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
     mbar_init(bar_drain, 1);
     *ab.flag = 0;
     *(ab.flag + 1) = 0;
+    reinterpret_cast<volatile int*>(smem + L::COUNT_OFF)[0] = splits;
     fence_barrier_init();
   }
   if (warp == 2) tmem_alloc(smem_u32(tmem_ptr), C::TMEM_COLS);
@@ -1141,7 +1155,6 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
   // the sequences in order of decreasing length (ties by index): items are taken in it
   int* order = reinterpret_cast<int*>(smem + L::ORDER_OFF);
   const bool sorted = seqlens != nullptr && B <= L::kMaxSortedB;
-  int count = splits;  // splits of every sequence
   if (sorted) {
     int* lens = reinterpret_cast<int*>(smem + L::LENS_OFF);
     for (int bb = threadIdx.x; bb < B; bb += blockDim.x) lens[bb] = seqlens[bb];
@@ -1155,13 +1168,17 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
       }
       order[r] = bb;
     }
-    // (by the loader warp, while warp 0 sorts; equal > 0 implies sorted)
-    if (warp == 1 && equal > 0) {
-      count = ragged_splits<D>(lens, B, Hkv, Skv, equal, splits, static_cast<int>(gridDim.x), lane);
-      if (blockIdx.x == 0 && lane == 0) sched[1] = static_cast<unsigned long long>(count);
+    // (by the last warp, which up to 64 sequences leave out of the sort; equal > 0 implies sorted)
+    if (warp == 2 && equal > 0) {
+      const int n = ragged_splits<D>(lens, B, Hkv, Skv, equal, splits, static_cast<int>(gridDim.x), lane);
+      if (lane == 0) {
+        reinterpret_cast<volatile int*>(smem + L::COUNT_OFF)[0] = n;
+        if (blockIdx.x == 0) sched[1] = static_cast<unsigned long long>(n);
+      }
     }
     __syncthreads();
   }
+  const int count = reinterpret_cast<const volatile int*>(smem + L::COUNT_OFF)[0];  // splits of every sequence
 
   if (warp == 1) {
     // ------------------------------------------------------------ loader (whole warp)
@@ -1181,6 +1198,7 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
     const long long per_seq = static_cast<long long>(Hkv) * count;
     const long long n_items = B * per_seq;
     int dynamic = -1;  // read from the first ticket once the first item is under way
+    const int lead = sorted && B > 1 ? L::kMergeLead : -1;
     long long item = blockIdx.x;
     int st = 0, nq = 0, skipped = -1;
     bool ok = true;
@@ -1235,7 +1253,6 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
             rec[4] = n_st;
             rec[5] = tok0;
             rec[6] = ntok;
-            rec[7] = count;
           }
           if constexpr (PAGED) {
             // pieces of min(page, 64) keys: a stage starts on a multiple of 64, so a piece
@@ -1274,6 +1291,13 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
             }
           }
           __syncwarp();
+          // one item for this CTA (not before the ring is full: the ticket is waited for here)
+          if (lead >= 0 && kk == 1 && j == max(n_st - 1 - lead, min(n_st, C::NSTAGE) - 1) && lane == 0) {
+            const long long next = static_cast<long long>(gridDim.x) +
+                                   (static_cast<uint32_t>(ticket >> 32) == kDecodeSchedTag
+                                        ? static_cast<uint32_t>(ticket) : blockIdx.x);
+            if (next >= n_items) asm volatile("griddepcontrol.launch_dependents;");
+          }
         }
       }
       if (!ok) break;
@@ -1288,10 +1312,10 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
       }
       item = __shfl_sync(0xffffffffu, item, 0);
     }
-    // Let the merge grid launch once every CTA has issued its last copy: early enough to hide
-    // the launch, and no waiting block takes an SM's issue slots or a CTA's place before that.
-    // GB300, us, against launching it at the start: B1 131072 keys 83.7 -> 83.0, B7 D64 3000 to
-    // 20000 keys 23.4 -> 22.4, B64 512 to 2048 keys 70.9 -> 70.2, short ones unchanged.
+    // Let the merge grid launch once every CTA has issued its last copy: no waiting block takes
+    // an SM's issue slots or a CTA's place before that.  GB300, us, against launching it at the
+    // start: B1 131072 keys 84.0 -> 83.4, B16 at 16 splits 68.6 -> 68.1, B4 4096 to 8192 keys at 8
+    // splits 26.0 -> 25.6.  (Earlier where one CTA works longest: see kMergeLead.)
     asm volatile("griddepcontrol.launch_dependents;");
     // the end record
     bool ended = false;
