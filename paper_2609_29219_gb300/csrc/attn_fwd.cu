@@ -2336,16 +2336,25 @@ cudaError_t launch_fwd_d(const FwdArgs& a, const KernelCtl& ctl, cudaStream_t st
   }
   static PerDeviceOnce configured_one;
   constexpr int kRows = FwdCfg<D>::NQT * FwdCfg<D>::BM;
-  // A plane's last item may have one query tile.  Running it as one pays off while the plane
-  // has few items (B8 H16/2 S300 causal: 15.2 -> 10.3 us); with many, the half item saved is
-  // less than the 2 % that the kernel with ONE is slower (B16 H8/1 S2000, 63 items: 178 us
-  // with the tile past the end computed, 185 without).  A causal last item is its longest.
-  const long long rows = static_cast<long long>(a.Sq) << fwd_pack_log2(a.Hq / a.Hkv, a.Sq);
-  const long long last = rows % kRows;
-  if (last > 0 && last <= FwdCfg<D>::BM && rows <= (a.causal ? 24 : 12) * static_cast<long long>(kRows))
-    return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D>, kRows, a, ctl, stream, configured_one);
-  return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D, false, 0, 0, false>, FwdCfg<D>::NQT * FwdCfg<D>::BM, a, ctl, stream,
-                                     configured2);
+  // A plane's last item may have one query tile.  Running it as one pays off where it is all of
+  // the plane (B7 H32 S128 D64 causal 10.2 -> 9.2 us, B12 H8 Sq 41 of 6461 62.8 -> 53.2), and where
+  // it is the last and longest of a causal launch of one round (B3 H6/3 S288 D128 8.7 -> 7.9, B10
+  // H12/1 S280 D64 8.3 -> 7.8).  Elsewhere the kernel with ONE is slower by more than the half
+  // item saves (B3 H16 S1038 D128 32.0 -> 34.9, B9 H16 S610 D64 25.2 -> 27.2, B5 H32 S2432 251 -> 261).
+  const int lg = fwd_pack_log2(a.Hq / a.Hkv, a.Sq);
+  const long long rows = static_cast<long long>(a.Sq) << lg, last = rows % kRows;
+  if (last > 0 && last <= FwdCfg<D>::BM) {
+    bool one = rows <= FwdCfg<D>::BM;
+    if (!one && a.causal) {
+      int dev = 0, sms = 0;
+      if (cudaGetDevice(&dev) == cudaSuccess &&
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+        one = (rows + kRows - 1) / kRows * ((a.B * a.Hq) >> lg) <= sms;
+    }
+    if (one) return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D>, kRows, a, ctl, stream, configured_one);
+  }
+  return launch_design<D, FwdCfg<D>, true>(attn_fwd_kernel<D, false, 0, 0, false>, kRows, a, ctl, stream,
+                                           configured2);
 }
 
 }  // namespace
@@ -2362,11 +2371,14 @@ int fwd_cluster_of(const FwdArgs& a) {
 }
 
 cudaError_t launch_fwd_varlen(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaStream_t stream) {
-  // Without a causal mask and with 8 query-tile pairs or more per sequence on average, the half
-  // item that a one-tile item saves is less than what its kernel costs (8 sequences of 1024 to
-  // 4096, H64/16 D64: 1022 us with ONE, 1005 without; H32/8 D128: 614 and 602).  A causal
-  // sequence's last item is its longest (12 of 1500 to 6000, H32/8: 1032 with, 1046 without).
-  if (!a.causal && a.total_q >= 8ll * 256 * a.B)
+  // Items of one query tile pay off where every sequence is one (B23 H8, 1 to 87 tokens, D64
+  // causal 12.8 -> 12.0 us) and, by a little, among the many items of long causal sequences, whose
+  // last is their longest (16 sequences of 1024 to 8192, H32/8 D128: 2319 -> 2298; 12 of 1500 to 6000
+  // 1046 -> 1032; ten other batches 0.97 to 1.02 times as fast).  Between these and without a causal
+  // mask their kernel costs more than the half items save: B24 H16, 17 to 136 tokens, causal 21.0 -> 22.3,
+  // B7 H32, 28 to 224, 16.9 -> 17.6 (but B14 H32, 50 to 396, D64 27.7 -> 25.7); B19 H64/16, 53 to 424, D64
+  // without a mask 60.1 -> 78.3.
+  if (a.max_seqlen_q > FwdCfg<128>::BM && !(a.causal && a.max_seqlen_q >= 1024))
     return a.D == 128 ? launch_varlen_d<128, false>(a, ctl, stream) : launch_varlen_d<64, false>(a, ctl, stream);
   return a.D == 128 ? launch_varlen_d<128, true>(a, ctl, stream) : launch_varlen_d<64, true>(a, ctl, stream);
 }

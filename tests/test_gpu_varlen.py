@@ -147,3 +147,25 @@ def test_cross_attention_lengths(loom):
     o, lse = run(loom, q, k, v, cq, ck, False)
     o_ref, lse_ref = oracle.attention_varlen(q, k, v, cq, ck, causal=False)
     assert_parity(o, o_ref, lse, lse_ref, "cross attention")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("lens,Hq,Hkv,causal", [
+    ([1, 128, 64, 127, 2, 33] * 20, 8, 2, True), ([1, 128, 64, 127, 2, 33] * 20, 8, 2, False),  # one tile each
+    ([2049, 2177, 2304, 2431, 2176], 4, 4, False),             # the last tile of 1 to 128 rows, or full
+    ([1024, 1025, 129, 1, 1153, 300, 128, 1280], 16, 2, True),  # items of one and of two tiles
+], ids=["short", "short_nc", "long_nc", "mixed"])
+def test_one_tile_items(loom, lens, Hq, Hkv, causal, D):
+    """Sequences whose last query tile has no second beside it, several items per CTA.  The
+    bound on the lengths picks the kernel and changes no bit."""
+    import torch
+    q, k, v, cq, ck = case(len(lens) + D, lens, lens, Hq, Hkv, D)
+    o, lse = run(loom, q, k, v, cq, ck, causal)
+    o_ref, lse_ref = oracle.attention_varlen(q, k, v, cq, ck, causal=causal)
+    assert_parity(o, o_ref, lse, lse_ref, f"{lens[:6]} D={D} causal={causal}")
+    args = [to_dev(q), to_dev(k), to_dev(v), torch.from_numpy(cq).cuda(), torch.from_numpy(ck).cuda()]
+    for bound in (512, 4096):  # either side of where the kernels change
+        if bound >= max(lens):
+            o2, lse2 = loom.loom_attn_fwd_varlen(*args, bound, causal=causal, return_lse=True)
+            loom.loom_attn_check_error()
+            assert np.array_equal(o2.float().cpu().numpy(), o) and np.array_equal(lse2.cpu().numpy(), lse)
