@@ -765,7 +765,12 @@ __device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars ba
 // tiles, and the partial results meet over distributed shared memory (split_epilogue).
 // ONE: items of one query tile may occur (the last of a plane); without them the roles need
 // no counts of their own per tile, worth 2 % on B4 H32 S2048 (169 against 173 us).
-template <int D, bool VARLEN = false, int SLOTS = 0, int SPLIT = 0, bool ONE = true>
+// DEFER (ragged batches): tile 1 releases the shared staging block an item later, once the
+// cursor has moved on, and not at all after the last item: released at once, the wait for the
+// store's read delays the walk to the next item or the end (GB300, D128, B1 H32/8 103 tokens
+// causal 8.0 -> 7.4 us, B16 H16 40 to 300 tokens 20.3 -> 19.8); not with the many items of long
+// causal sequences (16 of 1024 to 8192 tokens 2150 -> 2166).
+template <int D, bool VARLEN = false, int SLOTS = 0, int SPLIT = 0, bool ONE = true, bool DEFER = VARLEN && !ONE>
 __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
@@ -1060,7 +1065,9 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     const uint32_t my_bar_oe = bar_oe + 8 * t;
     const uint32_t stg_q =
         sbase + C::STG_OFF + static_cast<uint32_t>(C::SHARED_STG ? warp & 3 : warp) * (32 * D * 2);
+    const uint32_t stg_last = sbase + C::Q_OFF + C::Q_TILE_BYTES + static_cast<uint32_t>(warp & 3) * (32 * D * 2);
     // shared staging: tile 0's warp goes first, tile 1's after it, item by item
+    constexpr bool kDefer = C::SHARED_STG && DEFER;
     const uint32_t bar_mine = C::SHARED_STG ? bar_stg + 32 * t + 8 * (warp & 3) : 0;
     const uint32_t bar_peer = C::SHARED_STG ? bar_stg + 32 * (t ^ 1) + 8 * (warp & 3) : 0;
     const float c = p.c;
@@ -1074,6 +1081,10 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
     SeqCursor cur = VARLEN ? seq_cursor<kRows>(p) : SeqCursor{0, 0, 0};
     for (int r = 0, idx; ok && (idx = item_index_t<kRows, VARLEN>(p, r, cur, wk, n_wk)) >= 0; ++r) {
       const Item it = item_of(cur, idx);
+      if (kDefer && t == 1 && r > 0 && lane == 0) {
+        bulk_wait_group_read0();
+        mbar_arrive(bar_mine);
+      }
       const int row = (t == 0 ? it.q0 : it.q1) + row_in_tile;
       const int skv = VARLEN ? it.skv : p.Skv;
       const int offv = VARLEN ? it.skv - it.sq : off;
@@ -1101,11 +1112,19 @@ __global__ void __launch_bounds__(FwdCfg<D, SLOTS>::THREADS, 1)
           break;
         n_active += active;
       } else if (!ONE || my_tiles > 0) {
-        // shared staging: tile 0's release in this item, or tile 1's in the item before
+        // Shared staging: tile 0's release in this item, or tile 1's in the item before.  In the
+        // CTA's last item tile 1 stages in its Q tile, which nothing reads or loads any more, and
+        // waits for nobody: the turns cost a launch of one round 0.4 us (GB300, B3 H16/2 S128 D128
+        // 6.4 -> 5.9, B2 H64/16 S256 8.9 -> 8.4).  Not in a ragged batch, where the cursor would
+        // have to walk to the last sequence first.
+        bool last = false;
+        if constexpr (C::SHARED_STG && !VARLEN) last = item_index(p, r + 1, wk, n_wk) < 0;
+        const uint32_t stg = last && t == 1 ? stg_last : stg_q;
         if (!(ok = softmax_epilogue<D, VARLEN, !VARLEN>(
-                  o_tm, my_bar_o, my_n & 1, my_bar_oe, m_run, l_run, row, it.q_z, p, ab, &tm_o, stg_q,
-                  VARLEN ? it.qb : 0, VARLEN ? it.sq : 0, bar_mine, bar_peer, t == 1 ? n0 & 1 : (n1 - 1) & 1,
-                  C::SHARED_STG && (t == 1 ? !ONE || it.n_tiles0 > 0 : n1 > 0))))
+                  o_tm, my_bar_o, my_n & 1, my_bar_oe, m_run, l_run, row, it.q_z, p, ab, &tm_o, stg,
+                  VARLEN ? it.qb : 0, VARLEN ? it.sq : 0, last || (kDefer && t == 1) ? 0 : bar_mine, bar_peer,
+                  t == 1 ? n0 & 1 : (n1 - 1) & 1,
+                  C::SHARED_STG && (t == 1 ? !last && (!ONE || it.n_tiles0 > 0) : n1 > 0))))
           break;
       }
       cnt += my_tiles;
@@ -2059,7 +2078,7 @@ cudaError_t launch_dependent(bool dependent, Kernel kernel, int grid, int thread
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <int D, bool ONE>
+template <int D, bool ONE, bool DEFER>
 cudaError_t launch_varlen_d(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaStream_t stream) {
   using C = FwdCfg<D>;
   static PerDeviceOnce configured;
@@ -2071,9 +2090,9 @@ cudaError_t launch_varlen_d(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaSt
     return cudaErrorInvalidValue;
   int dev = 0;
   cudaGetDevice(&dev);
-  if (!configured.run(dev, [] {
-        return cudaFuncSetAttribute(attn_fwd_kernel<D, true, 0, 0, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    C::BYTES) == cudaSuccess;
+  const auto kernel = attn_fwd_kernel<D, true, 0, 0, ONE, DEFER>;
+  if (!configured.run(dev, [&] {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES) == cudaSuccess;
       }))
     return cudaErrorInvalidValue;
   FwdParams p;
@@ -2097,7 +2116,7 @@ cudaError_t launch_varlen_d(const FwdVarlenArgs& a, const KernelCtl& ctl, cudaSt
   constexpr int kRows = C::NQT * C::BM;
   const long long bound = static_cast<long long>(a.B) * a.Hq * ((a.max_seqlen_q + kRows - 1) / kRows);
   const int grid = static_cast<int>(bound > 0 && bound < sms ? bound : sms);
-  return launch_dependent(false, attn_fwd_kernel<D, true, 0, 0, ONE>, grid, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
+  return launch_dependent(false, kernel, grid, C::THREADS, C::BYTES, stream, mq, mk, mv, mo, p);
 }
 
 // Query heads of one kv head packed into a plane of the two-tile design (as a power of two):
@@ -2378,9 +2397,11 @@ cudaError_t launch_fwd_varlen(const FwdVarlenArgs& a, const KernelCtl& ctl, cuda
   // mask their kernel costs more than the half items save: B24 H16, 17 to 136 tokens, causal 21.0 -> 22.3,
   // B7 H32, 28 to 224, 16.9 -> 17.6 (but B14 H32, 50 to 396, D64 27.7 -> 25.7); B19 H64/16, 53 to 424, D64
   // without a mask 60.1 -> 78.3.
-  if (a.max_seqlen_q > FwdCfg<128>::BM && !(a.causal && a.max_seqlen_q >= 1024))
-    return a.D == 128 ? launch_varlen_d<128, false>(a, ctl, stream) : launch_varlen_d<64, false>(a, ctl, stream);
-  return a.D == 128 ? launch_varlen_d<128, true>(a, ctl, stream) : launch_varlen_d<64, true>(a, ctl, stream);
+  if (a.max_seqlen_q <= FwdCfg<128>::BM)
+    return a.D == 128 ? launch_varlen_d<128, true, true>(a, ctl, stream) : launch_varlen_d<64, true, false>(a, ctl, stream);
+  if (a.causal && a.max_seqlen_q >= 1024)
+    return a.D == 128 ? launch_varlen_d<128, true, false>(a, ctl, stream) : launch_varlen_d<64, true, false>(a, ctl, stream);
+  return a.D == 128 ? launch_varlen_d<128, false, true>(a, ctl, stream) : launch_varlen_d<64, false, true>(a, ctl, stream);
 }
 
 }  // namespace loom
