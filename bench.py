@@ -890,9 +890,9 @@ def run_ablation_sweep(torch, loom, dev, stream, args, peaks):
 
     # prefill: ring depth of the two-tile design (BN = 128 keys is fixed by the softmax layout)
     lens = synth.decode_lengths(0, 16, 4096, 8192)
-    prefill = [(Prefill("prefill", 4, 32, 32, 2048, 128, causal=False), (2, 3)),
-               (Prefill("prefill_causal", 4, 32, 32, 2048, 128, causal=True), (2, 3)),
-               (Prefill("long_prefill_d128", 1, 32, 8, 8192, 128, causal=True), (2, 3)),
+    prefill = [(Prefill("prefill", 4, 32, 32, 2048, 128, causal=False), (2, 3, 4)),
+               (Prefill("prefill_causal", 4, 32, 32, 2048, 128, causal=True), (2, 3, 4)),
+               (Prefill("long_prefill_d128", 1, 32, 8, 8192, 128, causal=True), (2, 3, 4)),
                (Prefill("long_prefill_d64", 1, 64, 16, 8192, 64, causal=True), (3, 6, 9, 10)),
                (Prefill("prefill_d64", 4, 32, 32, 2048, 64, causal=False), (3, 6, 9, 10))]
     for wl, depths in prefill:

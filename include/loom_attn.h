@@ -362,9 +362,9 @@ void loom_debug_prefill_design(int design);
  * the analytic model's constant and returns 1, or returns 0 (and restores the model's
  * constant) when that value is not compiled:
  * loom_debug_prefill_slots: the two-tile prefill's K/V ring depth for head dimension D
- *   (compiled beside the model's 3 at D = 128: 2; beside 10 at D = 64: 3, 6, 9; deeper
- *   rings do not fit in shared memory).  0 restores the model's, which at D = 128 runs with
- *   one slot more, in the memory that the query tiles' shared O staging leaves.
+ *   (compiled beside the model's 4 at D = 128: 2, 3; beside 10 at D = 64: 3, 6, 9; deeper
+ *   rings do not fit in shared memory).  A pinned depth, the model's too, runs one CTA per
+ *   work item.  0 restores the model's.
  * loom_debug_decode_stage_plan: the decode split kernel's keys per stage, ring stages and
  *   CTAs per SM (contiguous cache, D = 128, 4 query heads per kv head, split + merge form;
  *   compiled: 32x2x2, 32x3x2, 32x4x2, 64x2x2, 64x4x1, 128x2x1, 128x3x1 beside the model's

@@ -58,13 +58,13 @@ struct FwdCfg {
   static constexpr int NQT = kPlan.q_tiles;   // query tiles per CTA
   static constexpr int BN = kPlan.bn;         // keys per KV tile
   // At D = 128 both query tiles stage their O in one 32 KB block, in turn (see
-  // softmax_epilogue), and the 32 KB this frees are one more ring slot than the plan's 3: with
-  // three slots the MMA warp waited for K of every tile (about 300 of a pair of tile-steps'
+  // softmax_epilogue), and the 32 KB this frees are a fourth ring slot: with three
+  // slots the MMA warp waited for K of every tile (about 300 of a pair of tile-steps'
   // 2700 clocks in a clock trace).  GB300, same box, three slots against four: B4 H32 S2048
   // 190.7 -> 185.2 us, causal 116.9 -> 113.0, ragged causal batch (16 sequences of 1024 to
   // 8192) 2389 -> 2351.  D = 64 has ten slots and a block per tile.
   static constexpr bool SHARED_STG = D == 128;
-  static constexpr int NSLOT = SLOTS ? SLOTS : kPlan.kv_slots + (SHARED_STG ? 1 : 0);  // K/V ring slots
+  static constexpr int NSLOT = SLOTS ? SLOTS : kPlan.kv_slots;  // K/V ring slots
   static_assert(BM == 128 && NQT == 2, "warp roles assume two 128-row query tiles");
   static_assert(BN == 128, "softmax holds one S row of 128 fp32 in registers, P leaves in two 64-key halves");
   static_assert(kPlan.b_lm == 1 && NSLOT >= 2, "a K and a V slot at least");
@@ -89,7 +89,7 @@ struct FwdCfg {
   // H32 S2048: 184.4 -> 180.3 us); at D = 64, where the softmax bounds the step, it would
   // hold that S back (523 -> 529 us on H64/16 S8192 causal).  A ring of two slots cannot: that
   // V's slot is only released by this S.
-  static constexpr bool V_FIRST = D == 128 && NSLOT >= 3;
+  static constexpr bool V_FIRST = D == 128 && NSLOT >= 4;
   // ... and of a cluster that shares items: done, xdone, rdy[8], xf[8]
   static constexpr int NBAR = 4 + NSLOT + NKE + 11 + 8 + 18;
   static constexpr uint32_t TMEM_PTR_OFF = BAR_OFF + NBAR * 8;
@@ -2318,8 +2318,9 @@ cudaError_t launch_two_tile_slots(const FwdArgs& a, const KernelCtl& ctl, cudaSt
   *handled = true;
   constexpr int kRows = FwdCfg<D>::NQT * FwdCfg<D>::BM;
   if constexpr (D == 128) {
-    static PerDeviceOnce once2;
+    static PerDeviceOnce once2, once3;
     if (a.slots == 2) return launch_design<D, FwdCfg<D, 2>, true>(attn_fwd_kernel<D, false, 2>, kRows, a, ctl, stream, once2);
+    if (a.slots == 3) return launch_design<D, FwdCfg<D, 3>, true>(attn_fwd_kernel<D, false, 3>, kRows, a, ctl, stream, once3);
   } else {
     static PerDeviceOnce once3, once6, once9;
     if (a.slots == 3) return launch_design<D, FwdCfg<D, 3>, true>(attn_fwd_kernel<D, false, 3>, kRows, a, ctl, stream, once3);

@@ -98,9 +98,9 @@ struct FwdArgs {
 };
 
 // K/V ring depths of the two-tile prefill compiled beside the model's, for the block-size
-// ablation (D = 128: 2; D = 64: 3, 6, 9).
+// ablation (D = 128: 2, 3; D = 64: 3, 6, 9).
 inline bool fwd_slots_compiled(int D, int slots) {
-  return D == 128 ? slots == 2 : (slots == 3 || slots == 6 || slots == 9);
+  return D == 128 ? slots == 2 || slots == 3 : (slots == 3 || slots == 6 || slots == 9);
 }
 
 // Bytes of workspace the decode path needs for `splits` splits.

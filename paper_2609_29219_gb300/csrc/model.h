@@ -172,9 +172,11 @@ constexpr FwdPlan fwd_eval(const ArchDesc& a, int D, int design, int bn, int slo
   }
   p.t_iter_ns = heg_pipe(p.t_load_ns, body, 0.0, b_lm, b_ms);
   // resources (Eq. 8 constraints)
-  // Q tiles + K/V ring + an O staging tile per query tile (TMA-store epilogue) +
-  // barriers and alignment
-  p.smem_bytes = 2 * p.q_tiles * p.bm * D * 2 + slots * bn * D * 2 + 1024 + 256;
+  // Q tiles + K/V ring + O staging tiles (TMA-store epilogue) + barriers and alignment: one
+  // staging tile per query tile, but one for both in design 2 at D = 128, whose ring gains a
+  // slot by it (attn_fwd.cu, FwdCfg)
+  const int staging = design == 2 && D == 128 ? 1 : p.q_tiles;
+  p.smem_bytes = (p.q_tiles + staging) * p.bm * D * 2 + slots * bn * D * 2 + 1024 + 256;
   // design 4 keeps each tile's S and O adjacent at 32-column aligned bases (t * 160)
   p.tmem_cols = design == 1 ? 2 * bn + D : design == 2 ? 2 * (bn + D) : design == 3 ? 3 * bn + 2 * D
                                                                       : 3 * (bn + D);

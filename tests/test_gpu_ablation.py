@@ -36,7 +36,7 @@ def _qkv(seed, B, Hq, Hkv, Sq, Skv, D):
             synth.bf16_normal(seed, synth.STREAM_V, (B, Hkv, Skv, D)))
 
 
-@pytest.mark.parametrize("D,slots", [(128, 2), (64, 3), (64, 6), (64, 9)])
+@pytest.mark.parametrize("D,slots", [(128, 2), (128, 3), (64, 3), (64, 6), (64, 9)])
 @pytest.mark.parametrize("causal", [False, True])
 def test_prefill_ring_depths(loom, D, slots, causal):
     assert loom.loom_debug_prefill_slots(D, slots)
@@ -52,7 +52,7 @@ def test_prefill_ring_depths(loom, D, slots, causal):
 
 
 def test_prefill_rejects_depths_not_compiled(loom):
-    assert not loom.loom_debug_prefill_slots(128, 4)   # does not fit in shared memory
+    assert not loom.loom_debug_prefill_slots(128, 5)   # does not fit in shared memory
     assert not loom.loom_debug_prefill_slots(64, 11)
     assert loom.loom_debug_prefill_slots(128, 0)
 

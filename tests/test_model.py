@@ -228,3 +228,16 @@ def test_per_design_time_matches_the_choice(loom, D):
         assert (t < 0) == (loom.loom_model_fwd_plan_variant(D, d) is None)
         if t > 0:
             assert t >= loom.loom_model_fwd_time_us(*args) * (1 - 1e-9)  # the choice is the fastest
+
+
+def test_fwd_plan_ring_fills_shared_memory(loom):
+    """Two query tiles: at D = 128 one O staging tile for both leaves room for a fourth K/V
+    slot; the plan is what the kernel runs, and no deeper ring fits."""
+    for D, staging in ((64, 2), (128, 1)):
+        p = loom.loom_model_fwd_plan_variant(D, 2)
+        tile = p["bm"] * D * 2
+        assert p["smem_bytes"] == (2 + staging + p["kv_slots"]) * tile + 1280
+        assert p["smem_bytes"] + tile > 227 * 1024
+        assert loom.loom_debug_prefill_slots(D, p["kv_slots"]) and not loom.loom_debug_prefill_slots(D, p["kv_slots"] + 1)
+        assert loom.loom_debug_prefill_slots(D, 0)
+    assert loom.loom_model_fwd_plan(128)["kv_slots"] == 4
