@@ -57,12 +57,13 @@ struct FwdCfg {
   static constexpr int BM = kPlan.bm;         // rows per query tile (= TMEM lanes)
   static constexpr int NQT = kPlan.q_tiles;   // query tiles per CTA
   static constexpr int BN = kPlan.bn;         // keys per KV tile
-  // At D = 128 both query tiles stage their O in one 32 KB block, in turn (see
-  // softmax_epilogue), and the 32 KB this frees are a fourth ring slot: with three
-  // slots the MMA warp waited for K of every tile (about 300 of a pair of tile-steps'
-  // 2700 clocks in a clock trace).  GB300, same box, three slots against four: B4 H32 S2048
-  // 190.7 -> 185.2 us, causal 116.9 -> 113.0, ragged causal batch (16 sequences of 1024 to
-  // 8192) 2389 -> 2351.  D = 64 has ten slots and a block per tile.
+  // At D = 128 both query tiles stage their O in one 32 KB block, in turn (see softmax_epilogue),
+  // and the 32 KB this frees are a fourth ring slot: with three slots the MMA warp waits for K of
+  // every tile.  GB300, same box, us a pass, three slots against four in the kernel as it is
+  // otherwise: B4 H32 S2048 213 -> 182, causal 126.6 -> 113.7, ragged causal batch (16 sequences
+  // of 1024 to 8192) 2598 -> 2308.  (Most of that is this kernel's: three slots with a staging
+  // block per tile and a commit per K and V tile ran 192, 123 and 2469.)  D = 64 has ten slots and
+  // a block per tile.
   static constexpr bool SHARED_STG = D == 128;
   static constexpr int NSLOT = SLOTS ? SLOTS : kPlan.kv_slots;  // K/V ring slots
   static_assert(BM == 128 && NQT == 2, "warp roles assume two 128-row query tiles");
@@ -85,10 +86,11 @@ struct FwdCfg {
   // together by the commit behind the last S of K number n, on barrier n % NKE.
   static constexpr int NKE = (NSLOT + 1) / 2;
   // The MMA warp waits for the next V before it issues tile 1's next S, while P.V keeps the
-  // tensor pipe busy, and not after it, when the pipe runs dry meanwhile: at D = 128 +2.3 % (B4
-  // H32 S2048: 184.4 -> 180.3 us); at D = 64, where the softmax bounds the step, it would
-  // hold that S back (523 -> 529 us on H64/16 S8192 causal).  A ring of two slots cannot: that
-  // V's slot is only released by this S.
+  // tensor pipe busy, and not after it, when the pipe runs dry meanwhile.  GB300, us a pass, after /
+  // before, D = 128: B4 H32 S2048 185.5 / 183.2, causal 115.1 / 114.8 (within the spread), ragged
+  // causal batch 2344 / 2332; at D = 64, where the softmax bounds the step, it would hold that S back
+  // (523 -> 529 on H64/16 S8192 causal).  A ring of three slots or two cannot: that V's slot is only
+  // released by this S, or by the S before it.
   static constexpr bool V_FIRST = D == 128 && NSLOT >= 4;
   // ... and of a cluster that shares items: done, xdone, rdy[8], xf[8]
   static constexpr int NBAR = 4 + NSLOT + NKE + 11 + 8 + 18;
@@ -338,9 +340,9 @@ __device__ __forceinline__ bool softmax_step(uint32_t s_tm, uint32_t o_tm, uint3
   if (kbase + BN > limit) {
     // A diagonal or ragged tile's step is issue-bound, and its length is on the item's
     // critical path: each key tests a constant bit of its chunk's word of visible keys
-    // instead of comparing its number with the limit.  GB300, same box, in us: B4 H32 S2048
-    // D128 causal 121.8 -> 116.0, D64 S8192 causal 544 -> 536, ragged causal batch (16
-    // sequences of 1024 to 8192) 2431 -> 2363, Sq 515 of Skv 3001 causal 38.7 -> 37.7.
+    // instead of comparing its number with the limit.  GB300, same box, us a pass: B4 H32 S2048
+    // D128 causal 119.6 -> 116.2, D64 S8192 causal 532.6 -> 524.4, ragged causal batch (16
+    // sequences of 1024 to 8192) 2363 -> 2321.
 #pragma unroll
     for (int g = 0; g < BN / 32; ++g) {
       const int n = limit - kbase - 32 * g;  // visible keys of the chunk
@@ -430,6 +432,11 @@ __device__ __forceinline__ bool softmax_step(uint32_t s_tm, uint32_t o_tm, uint3
   return true;
 }
 
+// Where the log-sum-exp of row `row` of plane q_z of packed heads is stored.
+__device__ __forceinline__ size_t packed_lse_row(const FwdParams& p, int q_z, int row) {
+  return ((static_cast<size_t>(q_z) << p.pack_log2) + (row & ((1 << p.pack_log2) - 1))) * p.Sq + (row >> p.pack_log2);
+}
+
 // Epilogue of one query row (this thread's TMEM lane): wait for the last P.V (bar_o,
 // par_o), read O from TMEM into registers as bf16 O / l and hand the O columns back to
 // the MMA warp at once (bar_oe); then write the row into this warp's staging block in
@@ -447,10 +454,6 @@ __device__ __forceinline__ bool softmax_step(uint32_t s_tm, uint32_t o_tm, uint3
 // item boundary, where this warp waits for the next item's first S anyway.
 // PACKED: O rows are rows of a plane of packed heads (FwdParams::pack_log2; the 32 rows of
 // a warp are one box of the 4-D output map).
-__device__ __forceinline__ size_t packed_lse_row(const FwdParams& p, int q_z, int row) {
-  return ((static_cast<size_t>(q_z) << p.pack_log2) + (row & ((1 << p.pack_log2) - 1))) * p.Sq + (row >> p.pack_log2);
-}
-
 template <int D, bool VARLEN = false, bool PACKED = false>
 __device__ __forceinline__ bool softmax_epilogue(uint32_t o_tm, uint32_t bar_o, uint32_t par_o,
                                                  uint32_t bar_oe, float m_run, float l_run,
@@ -575,21 +578,6 @@ __device__ __forceinline__ void prefetch_item_l2(const CUtensorMap* tm_q, const 
   }
 }
 
-// Epilogue of one query row when a cluster of S CTAs shares the item.  Each CTA holds the
-// row's (m, l) and unnormalised O over its own KV tiles; CTA q of the cluster finishes
-// columns [q D / S, (q + 1) D / S) of both query tiles.  So the warp sends, for every other
-// CTA, its rows' (m, l) and those columns of O (fp32) into that CTA's Q tiles and K slots
-// (the even ring slots) -- idle once that CTA's last S of the item is done, which it
-// announces on bar_rdy[its rank] a tile-step before it needs the partials -- waits for
-// the S - 1 partials of its own rows (bar_xf[warp]), and sums the S partials in rank order
-// (the result does not depend on timing), O = sum 2^(m_s - M) O_s / sum 2^(m_s - M) l_s.
-// Layout (of the 16-byte units, see partial_at), per source CTA: float4 chunk c of row r at (c * 256 + r) * 16 (a
-// warp's 32 rows are contiguous: no bank conflicts on either side), then (m, l) per row.
-// has_tiles: this CTA walked KV tiles of the row's tile; active: the item has that tile.
-// The finished columns go through the warp's staging block (4 KB) so that a warp stores
-// whole rows' pieces: stored straight from the row threads, 32 rows per instruction, the
-// stores alone took 2 us of the exchange's 7.  Not inlined: its registers would spill
-// values of the softmax loop around it.
 // Byte `off` of the partials' space: the Q tiles and ring slot 0, which follow one another,
 // then ring slots 2, 4, ...
 template <class C>
@@ -612,6 +600,21 @@ struct SplitRow {
 struct SplitBars {
   uint32_t o, oe, rdy, xf, xdone;
 };
+// Epilogue of one query row when a cluster of S CTAs shares the item.  Each CTA holds the
+// row's (m, l) and unnormalised O over its own KV tiles; CTA q of the cluster finishes
+// columns [q D / S, (q + 1) D / S) of both query tiles.  So the warp sends, for every other
+// CTA, its rows' (m, l) and those columns of O (fp32) into that CTA's Q tiles and K slots
+// (the even ring slots) -- idle once that CTA's last S of the item is done, which it
+// announces on bar_rdy[its rank] a tile-step before it needs the partials -- waits for
+// the S - 1 partials of its own rows (bar_xf[warp]), and sums the S partials in rank order
+// (the result does not depend on timing), O = sum 2^(m_s - M) O_s / sum 2^(m_s - M) l_s.
+// Layout (of the 16-byte units, see partial_at), per source CTA: float4 chunk c of row r at (c * 256 + r) * 16 (a
+// warp's 32 rows are contiguous: no bank conflicts on either side), then (m, l) per row.
+// has_tiles: this CTA walked KV tiles of the row's tile; active: the item has that tile.
+// The finished columns go through the warp's staging block (4 KB) so that a warp stores
+// whole rows' pieces: stored straight from the row threads, 32 rows per instruction, the
+// stores alone took 2 us of the exchange's 7.  Not inlined: its registers would spill
+// values of the softmax loop around it.
 template <int D, int S>
 __device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars bar, uint32_t o_tm, uint32_t sbase,
                                             uint32_t stg, int warp, int rank, const KernelCtl ctl, const Abort ab) {
@@ -764,7 +767,8 @@ __device__ __noinline__ bool split_epilogue(const SplitRow r, const SplitBars ba
 // SPLIT = S > 0: a cluster of S CTAs (2, 4 or 8) shares every item, each CTA walking 1/S of its KV
 // tiles, and the partial results meet over distributed shared memory (split_epilogue).
 // ONE: items of one query tile may occur (the last of a plane); without them the roles need
-// no counts of their own per tile, worth 2 % on B4 H32 S2048 (169 against 173 us).
+// no counts of their own per tile (GB300, with / without, a launch among captured ones: B4 H32
+// S2048 172 / 168 us, causal 109.5 / 105.8; a pass, H64/16 S8192 D64 causal 539 / 523).
 // DEFER (ragged batches): tile 1 releases the shared staging block an item later, once the
 // cursor has moved on, and not at all after the last item: released at once, the wait for the
 // store's read delays the walk to the next item or the end (GB300, D128, B1 H32/8 103 tokens
