@@ -21,22 +21,29 @@ def loom():
     return m
 
 
-# B, Hq, Hkv, Sq, Skv, D, causal: clusters of 2 with a one-tile item last in its plane; of 4
-# with 1000 + 1 rows of G = 2; of 8 with a handful of rows; several items per cluster; a
-# share that ends before tile 0's diagonal; groups that are no power of two; no causal mask
-SHAPES = [
+# B, Hq, Hkv, Sq, Skv, D, causal.  CLUSTERED, one item per cluster: of 2 with a one-tile item last
+# in its plane; of 2 or 4 with 1400 rows of G = 2; of 8 with a handful of rows; a share that ends
+# before tile 0's diagonal; groups that are no power of two; no causal mask
+CLUSTERED = [
     (1, 32, 8, 515, 3001, 128, True), (2, 6, 3, 700, 2000, 128, True), (1, 8, 1, 3, 4100, 128, True),
     (1, 8, 1, 300, 2049, 64, True), (1, 8, 8, 2048, 2048, 128, True), (1, 4, 4, 1500, 1500, 64, True),
-    (1, 6, 1, 130, 2300, 128, False), (2, 4, 4, 129, 5000, 64, False), (1, 32, 1, 65, 1025, 128, True),
-    (1, 12, 1, 129, 4096, 64, True), (3, 16, 4, 257, 2600, 128, False),
-    # a last item of one tile among few of its plane, and among many (computed as two)
-    (9, 16, 2, 300, 300, 64, True), (2, 4, 4, 3400, 300, 128, False),
+    (1, 6, 1, 130, 2300, 128, False), (2, 4, 4, 129, 5000, 64, False), (1, 12, 1, 129, 4096, 64, True),
+    (3, 16, 4, 257, 2600, 128, False),
+]
+SHAPES = CLUSTERED + [
+    # a last item of one tile: run as one in a causal launch of one round and where it is all of
+    # its plane, computed as two in more rounds and without a causal mask
+    (1, 32, 1, 65, 1025, 128, True), (3, 6, 3, 288, 288, 128, True), (10, 12, 1, 280, 280, 64, True),
+    (7, 32, 32, 128, 128, 64, True), (40, 8, 8, 50, 170, 128, False), (9, 16, 2, 300, 300, 64, True),
+    (2, 4, 4, 3400, 300, 128, False), (3, 16, 2, 128, 128, 128, False),
 ]
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,Sq,Skv,D,causal", SHAPES)
 def test_few_items(loom, B, Hq, Hkv, Sq, Skv, D, causal):
     import torch
+    clustered = (B, Hq, Hkv, Sq, Skv, D, causal) in CLUSTERED
+    assert (loom.loom_attn_fwd_cluster(B, Hq, Hkv, Sq, Skv, D, causal) > 1) == clustered
     q = synth.bf16_normal(1, synth.STREAM_Q, (B, Hq, Sq, D))
     k = synth.bf16_normal(1, synth.STREAM_K, (B, Hkv, Skv, D))
     v = synth.bf16_normal(1, synth.STREAM_V, (B, Hkv, Skv, D))
@@ -97,6 +104,7 @@ def test_extreme_scores_across_shares(loom):
     kf = (k.astype(np.uint32) << 16).view(np.float32).copy()
     kf[:, :, :700] *= 60.0
     k = synth.f32_to_bf16(kf)
+    assert loom.loom_attn_fwd_cluster(B, Hq, Hkv, Sq, Skv, D) > 1
     o, lse = loom.loom_attn_fwd(to_dev(q), to_dev(k), to_dev(v), return_lse=True)
     loom.loom_attn_check_error()
     o_ref, lse_ref = oracle.attention(q, k, v)
@@ -106,7 +114,7 @@ def test_extreme_scores_across_shares(loom):
 NAN, INF = 0x7FC0, 0x7F80  # bf16 bits
 
 
-# The shape's clusters: of 2 with a first item whose tile 0 falls to one CTA, of 2, of 8
+# Clusters of 2 with a first item whose tile 0 falls to one CTA, of 4, of 4
 @pytest.mark.parametrize("tensor,pos,bits", [
     ("q", 5, NAN), ("q", -1, NAN), ("k", 0, NAN), ("k", 777, NAN), ("k", -1, NAN), ("k", 300, INF), ("v", 0, NAN),
     ("v", 900, INF), ("v", -1, NAN)])
@@ -125,6 +133,7 @@ def test_nan_and_infinity(loom, steep, tensor, pos, bits, B, Hq, Hkv, Sq, Skv, D
         k = synth.f32_to_bf16(kf)
     {"q": q, "k": k, "v": v}[tensor][0, 0, pos, 3] = bits
     qd, kd, vd = to_dev(q), to_dev(k), to_dev(v)
+    assert loom.loom_attn_fwd_cluster(B, Hq, Hkv, Sq, Skv, D, causal) > 1
     o, lse = loom.loom_attn_fwd(qd, kd, vd, causal=causal, return_lse=True)
     loom.loom_debug_prefill_slots(D, 2 if D == 128 else 9)  # a pinned ring depth runs one CTA per item
     try:
@@ -151,6 +160,7 @@ def test_timeout_in_a_cluster_is_reported(loom, D):
     q = synth.bf16_normal(3, synth.STREAM_Q, (B, Hq, Sq, D))
     k = synth.bf16_normal(3, synth.STREAM_K, (B, Hkv, Skv, D))
     v = synth.bf16_normal(3, synth.STREAM_V, (B, Hkv, Skv, D))
+    assert loom.loom_attn_fwd_cluster(B, Hq, Hkv, Sq, Skv, D) > 1
     qd, kd, vd = to_dev(q), to_dev(k), to_dev(v)
     loom.loom_attn_check_error()
     loom.loom_debug_set_timeout_ns(50_000_000)
