@@ -23,6 +23,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "gemm.h"
 #include "gemm_model.h"
@@ -473,37 +474,50 @@ __global__ void __launch_bounds__(C::SPLIT_THREADS, 1)
     constexpr int kChunks = BN / 4;  // 16-byte chunks of a partial row
     const int all = valid * kChunks;  // chunks of C's rows, dealt evenly to the cluster's CTAs
     const int log_s = __ffs(S) - 1;
+    int base = (all * static_cast<int>(rank)) >> log_s;
     const int last = (all * (static_cast<int>(rank) + 1)) >> log_s;
-    // kBatch chunks per thread at a time: a remote read's latency, not its bytes, is what a
-    // chunk on its own waits for
-    constexpr int kBatch = 4;
-    for (int i0 = ((all * static_cast<int>(rank)) >> log_s) + static_cast<int>(threadIdx.x); i0 < last;
-         i0 += 128 * kBatch) {
+    // A remote read's latency, not its bytes, is what a chunk waits for, so a thread has eight
+    // reads in flight: as many partials of one chunk as there are (up to eight), so that the
+    // cluster's CTAs do not all read one peer's memory at once, and then of two or four chunks of
+    // its own where they are there.  GB300, us, one chunk at a time / four chunks whether there are as
+    // many or not, two partials ahead / so: M 153 N 384 K 3968, 16 splits, 7.2 / 9.3 / 7.0, M 298 N 512
+    // K 3712, 8 splits, 7.6 / 8.6 / 7.5; M 16 N 6144 K 4096, 4 splits, a pass - / 12.4 / 12.1.
+    auto reduce = [&](auto batch) {
+      constexpr int kBatch = decltype(batch)::value, kAhead = 8 / kBatch;
       float4 acc[kBatch];
       uint32_t off[kBatch];
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
-        const int i = min(i0 + 128 * u, last - 1);  // (past the end: read again, not stored)
+        const int i = min(base + static_cast<int>(threadIdx.x) + 128 * u, last - 1);  // (past the end: not stored)
         const int r = i / kChunks, j = i % kChunks;
         off[u] = sbase + static_cast<uint32_t>(r) * kRowBytes + ((static_cast<uint32_t>(j) ^ (r & 7)) << 4);
         acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-#pragma unroll 2
-      for (int s = 0; s < S; ++s) {
-        float4 v[kBatch];
+#pragma unroll 1
+      for (int s0 = 0; s0 < S; s0 += kAhead) {
+        float4 v[kAhead][kBatch];
 #pragma unroll
-        for (int u = 0; u < kBatch; ++u) v[u] = ld_dsmem_f4(map_shared_rank(off[u], static_cast<uint32_t>(s)));
+        for (int k = 0; k < kAhead; ++k)
+          if (s0 + k < S) {
 #pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          acc[u].x += v[u].x;
-          acc[u].y += v[u].y;
-          acc[u].z += v[u].z;
-          acc[u].w += v[u].w;
-        }
+            for (int u = 0; u < kBatch; ++u)
+              v[k][u] = ld_dsmem_f4(map_shared_rank(off[u], static_cast<uint32_t>(s0 + k)));
+          }
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k)
+          if (s0 + k < S) {
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+              acc[u].x += v[k][u].x;
+              acc[u].y += v[k][u].y;
+              acc[u].z += v[k][u].z;
+              acc[u].w += v[k][u].w;
+            }
+          }
       }
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
-        const int i = i0 + 128 * u;
+        const int i = base + static_cast<int>(threadIdx.x) + 128 * u;
         const int grow = tm * C::BM + i / kChunks, gcol = tn * BN + (i % kChunks) * 4;
         if (i < last && gcol < p.N) {  // N % 8 == 0: the 4 columns are all inside C
           uint2 w;
@@ -512,6 +526,16 @@ __global__ void __launch_bounds__(C::SPLIT_THREADS, 1)
           *reinterpret_cast<uint2*>(p.c + static_cast<size_t>(grow) * p.N + gcol) = w;
         }
       }
+      base += 128 * kBatch;
+    };
+    while (base < last) {
+      const int left = last - base;
+      if (S == 2 && left > 256)
+        reduce(std::integral_constant<int, 4>{});
+      else if (S <= 4 && left > 128)
+        reduce(std::integral_constant<int, 2>{});
+      else
+        reduce(std::integral_constant<int, 1>{});
     }
   }
 
