@@ -949,13 +949,13 @@ template <int D>
 struct DecodeTcPersistCfg {
   using C = DecodeTcCfg<D>;
   static constexpr int kMaxSortedB = kMaxRaggedB;         // sequences sorted by length
-  // Stages that a CTA has still to issue when it lets the merge grid launch, where it has one
-  // item of a batch of several sequences: the CTA of the longest works on alone, and after its
-  // last copy too little time is left to hide the launch.  GB300, us, launched at the start / at
-  // 0 / 10 / 24 stages: lengths from half the longest up, B32 H64/8 2977 keys 63.4 / 64.2 / 63.0 /
-  // 62.8, B18 H64/8 3049 keys 39.4 / 40.0 / 39.3 / 39.5; one length, B32 H64/8 2977 keys 70.1 / 70.5 /
-  // 70.5 / 70.5.  Several items per CTA end together: 0 is better (B16 4096 to 8192 keys of 16 in a
-  // page at 12 splits 71.2, at 10 stages 72.0).
+  // Stages that a CTA has still to issue when it lets the merge grid launch, where no CTA has more
+  // than one item, longer than this, of several sequences: the CTA of the longest works on alone,
+  // and after its last copy too little time is left to hide the launch.  GB300, us, launched at the
+  // start / at 0 / 10 / 24 stages: lengths from half the longest up, B32 H64/8 2977 keys 63.4 / 64.2 / 63.0 /
+  // 62.8, B18 H64/8 3049 keys 39.4 / 40.0 / 39.3 / 39.5; one length, B32 H64/8 2977 keys 70.1 / 70.5 / 70.5 /
+  // 70.5.  Several items per CTA end together: 0 is better (B16 4096 to 8192 keys of 16 in a page at
+  // 12 splits 71.2, at 10 stages 72.0); so do short ones (B8 672 keys at 4 splits 11.7, at once 12.0).
   static constexpr int kMergeLead = 10;
   static constexpr uint32_t Q_BOX_BYTES = C::MAX_G * 128;  // up to 32 heads x 64 dims
   static constexpr uint32_t Q_OFF = C::NSTAGE * C::STAGE_BYTES;
@@ -1198,7 +1198,6 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
     const long long per_seq = static_cast<long long>(Hkv) * count;
     const long long n_items = B * per_seq;
     int dynamic = -1;  // read from the first ticket once the first item is under way
-    const int lead = sorted && B > 1 ? L::kMergeLead : -1;
     long long item = blockIdx.x;
     int st = 0, nq = 0, skipped = -1;
     bool ok = true;
@@ -1234,7 +1233,10 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
         ++nq;
         const int n_st = (t_end - t_begin + C::T - 1) / C::T;
         const int kv_z = b * Hkv + hk;
+        // (the merge grid's launch; no CTA has a second item: see kMergeLead)
+        const int early = sorted && B > 1 && n_items <= gridDim.x ? n_st - 1 - L::kMergeLead : -1;
         for (int j = 0; j < n_st; ++j, ++st) {
+          if (j == early) asm volatile("griddepcontrol.launch_dependents;");
           const int s = st % C::NSTAGE;
           if (!(ok = mbar_wait_warp(bar_empty + 8 * s, ((st / C::NSTAGE) & 1) ^ 1, ctl, ab))) break;
           if (ctl.inject == 1 && st == 1) {  // test hook: never fill this stage
@@ -1291,13 +1293,6 @@ __global__ void __launch_bounds__(DecodeTcCfg<D>::THREADS, 2)
             }
           }
           __syncwarp();
-          // one item for this CTA (not before the ring is full: the ticket is waited for here)
-          if (lead >= 0 && kk == 1 && j == max(n_st - 1 - lead, min(n_st, C::NSTAGE) - 1) && lane == 0) {
-            const long long next = static_cast<long long>(gridDim.x) +
-                                   (static_cast<uint32_t>(ticket >> 32) == kDecodeSchedTag
-                                        ? static_cast<uint32_t>(ticket) : blockIdx.x);
-            if (next >= n_items) asm volatile("griddepcontrol.launch_dependents;");
-          }
         }
       }
       if (!ok) break;
